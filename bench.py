@@ -136,7 +136,7 @@ def _traffic_per_launch(kernel: str):
 KERNEL_SOURCES = {
     "fft_strided_tma_L512": ["tfft_tma.cu", "tfft_tma.cuh", "tfft_tiles.cuh", "tfft_common.cuh",
                              "tfft_internal.h", "tfft_device_cache.h"],
-    "fft_contig_L512": ["tfft_spec.cu", "tfft_spec_table.h", "tfft_tiles.cuh", "tfft_common.cuh",
+    "fft_contig_L512": ["tfft_spec_pass.cuh", "tfft_spec_table.h", "tfft_tiles.cuh", "tfft_common.cuh",
                         "tfft_internal.h", "tfft_device_cache.h"],
 }
 

@@ -20,7 +20,18 @@ LIB = os.path.join(PKG, "libtfft.so")
 
 SOURCES = ["tfft_kernels.cu", "tfft_spec.cu", "tfft_spec_real.cu", "tfft_tma.cu", "tfft_noalloc.cu", "tfft_pointwise.cu", "tfft_batch.cu", "tfft_tc.cu", "tfft_tc_strided.cu", "tfft_blue.cu", "tfft_plan.cpp", "tfft_exchange.cpp",
            "tfft_tmageo.cpp", "tfft_exec.cpp", "tfft_hostio.cpp", "tfft_batch_host.cpp"]
+# the specialised passes, one object per part of their table (kSpecParts in tfft_spec_pass.cuh)
+PARTS = {"tfft_spec_part.cu": [("TFFT_SPEC_PART", k) for k in range(11)]}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
+
+
+def _units():
+    """(source file, object name, extra flags) of every translation unit."""
+    for src in SOURCES:
+        yield src, src + ".o", []
+    for src, parts in PARTS.items():
+        for name, k in parts:
+            yield src, f"{src}.{k}.o", [f"-D{name}={k}"]
 
 
 def nvcc() -> str:
@@ -50,12 +61,12 @@ def build(verbose: bool = False, force: bool = False, ptxas_verbose: bool = Fals
     headers = [os.path.join(CSRC, h) for h in os.listdir(CSRC) if h.endswith((".h", ".cuh", ".map"))]
     headers.append(os.path.join(INCLUDE, "tfft.h"))
     procs, objs = [], []
-    for src in SOURCES:
+    for src, oname, extra in _units():
         path = os.path.join(CSRC, src)
-        obj = os.path.join(BUILD, src + ".o")
+        obj = os.path.join(BUILD, oname)
         objs.append(obj)
         if force or _stale(obj, [path] + headers):
-            cmd = [nvcc(), "-c", path, "-o", obj] + _flags(ptxas_verbose)
+            cmd = [nvcc(), "-c", path, "-o", obj] + _flags(ptxas_verbose) + extra
             if src.endswith(".cpp"):
                 cmd[1:1] = ["-x", "c++"]
             if verbose:

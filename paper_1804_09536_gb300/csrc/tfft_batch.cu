@@ -146,7 +146,7 @@ __device__ int tma_item(const BatchSeg& S, int64_t t0, int64_t t1, float2* smem,
 #pragma unroll
           for (int r = 0; r < R; ++r) v[q * R + r] = cur[(jt + q * T + r * (L / R)) * W + cx];
       }
-      spec_stage<L, E, R, Ns>(v, jt, a.tw);
+      spec_stage<L, T, R, Ns>(v, jt, a.tw);
     });
     constexpr int RL = radix_at<NST - 1, Rs...>();
     __syncthreads();
@@ -179,9 +179,9 @@ __device__ int tma_item(const BatchSeg& S, int64_t t0, int64_t t1, float2* smem,
 template <int KIND, int L, int E, int BW, int... Rs>
 __device__ __forceinline__ void run_tile(const BatchSeg& S, int64_t tile, float2* smem, int tid) {
   if constexpr (KIND == 0)
-    contig_tile<L, E, BW, true, Rs...>(S.ca, tile, smem, tid % (L / E), tid / (L / E));
+    contig_tile<L, L / E, BW, true, Rs...>(S.ca, tile, smem, tid % (L / E), tid / (L / E));
   else
-    strided_tile<L, E, BW, true, Rs...>(S.sa, tile, smem, tid % BW, tid / BW, tid);
+    strided_tile<L, L / E, BW, true, Rs...>(S.sa, tile, smem, tid % BW, tid / BW, tid);
 }
 
 // Segments whose first-item table fits shared memory use it for the lookup.

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__((M / E) * B, min_blocks(E, (M / E) * B, 512))
         }
         v[q * R0 + r] = x;
       }
-    line_stages<M, E, Rs...>(v, sl, jt, b.twm);
+    line_stages<M, T, Rs...>(v, sl, jt, b.twm);
     // filter, conjugated for the inverse, then back to the first stage's order
     line_sync<T>();
 #pragma unroll
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__((M / E) * B, min_blocks(E, (M / E) * B, 512))
     for (int q = 0; q < E / R0; ++q)
 #pragma unroll
       for (int r = 0; r < R0; ++r) v[q * R0 + r] = sl[padp<P>(jt + q * T + r * (M / R0))];
-    line_stages<M, E, Rs...>(v, sl, jt, b.twm);
+    line_stages<M, T, Rs...>(v, sl, jt, b.twm);
 #pragma unroll
     for (int q = 0; q < E / RL; ++q)
 #pragma unroll
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(W * (M / E), min_blocks(E, W * (M / E), 768))
         }
         v[q * R0 + r] = x;
       }
-    strided_stages<M, E, W, Rs...>(v, smem, cx, jt, b.twm);
+    strided_stages<M, T, W, Rs...>(v, smem, cx, jt, b.twm);
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < E / RL; ++q)
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(W * (M / E), min_blocks(E, W * (M / E), 768))
     for (int q = 0; q < E / R0; ++q)
 #pragma unroll
       for (int r = 0; r < R0; ++r) v[q * R0 + r] = smem[(jt + q * T + r * (M / R0)) * W + cx];
-    strided_stages<M, E, W, Rs...>(v, smem, cx, jt, b.twm);
+    strided_stages<M, T, W, Rs...>(v, smem, cx, jt, b.twm);
 #pragma unroll
     for (int q = 0; q < E / RL; ++q)
 #pragma unroll

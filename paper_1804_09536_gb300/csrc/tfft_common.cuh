@@ -248,6 +248,163 @@ struct Dft<32> {
   }
 };
 
+// ------------------------------------------------------------ composed DFTs
+//
+// The other radices: odd primes by their cosine / sine sums, composite ones
+// by the prime factor map (coprime factors, no twiddles) or a Cooley-Tukey
+// step with constant twiddles.  Every constant is formed in double precision
+// at compile time.
+
+// cos and sin of 2 pi m / n: m reduced to the first octant as an integer,
+// then the Taylor series on [0, pi / 4] (below 2^-60 after these terms).
+struct CosSin {
+  double c, s;
+};
+constexpr CosSin cos_sin(int m, int n) {
+  m %= n;
+  // angle = (pi / 4) (8 m / n): octant, and the remainder's distance
+  const int o = 8 * m / n;
+  const int up = (o & 1) ? (o + 1) * n - 8 * m : 8 * m - o * n;  // distance to the even octant edge, in n-ths of pi / 4
+  const double x = 0.78539816339744830961566 * (double)up / (double)n;
+  double c = 0.0, s = 0.0, t = 1.0;
+  for (int k = 0; k < 24; ++k) {  // t = x^k / k!
+    if (k & 1) s += (k & 2) ? -t : t;
+    else c += (k & 2) ? -t : t;
+    t = t * x / (double)(k + 1);
+  }
+  // edge e = ((o + 1) / 2) quarter turns; x is measured from it, forward for even octants, backward for odd ones
+  if (o & 1) s = -s;
+  switch (((o + 1) / 2) & 3) {
+    case 0: return CosSin{c, s};
+    case 1: return CosSin{-s, c};
+    case 2: return CosSin{-c, -s};
+    default: return CosSin{s, -c};
+  }
+}
+
+// exp(-2 pi i M / N) as a pair of compile-time floats.
+template <int N, int M>
+struct Root {
+  static constexpr float re = (float)cos_sin(M % N, N).c;
+  static constexpr float im = (float)-cos_sin(M % N, N).s;
+};
+
+template <int I>
+struct IntC {
+  static constexpr int value = I;
+};
+template <int I, int N, class F>
+TFFT_HD void unrolled(F&& f) {
+  if constexpr (I < N) {
+    f(IntC<I>{});
+    unrolled<I + 1, N>(f);
+  }
+}
+
+// Odd prime P: with t_k = v_k + v_{P-k}, u_k = v_k - v_{P-k}, k <= (P - 1) / 2,
+// X_j, X_{P-j} = v_0 + sum t_k cos(2 pi j k / P) -+ i sum u_k sin(2 pi j k / P).
+template <int P>
+struct DftPrime {
+  TFFT_HD static void run(float2* v) {
+    constexpr int H = (P - 1) / 2;
+    float2 t[H], u[H];
+    const float2 a = v[0];
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+      t[k] = cadd(v[k + 1], v[P - 1 - k]);
+      u[k] = csub(v[k + 1], v[P - 1 - k]);
+    }
+    float2 sum = a;
+#pragma unroll
+    for (int k = 0; k < H; ++k) sum = cadd(sum, t[k]);
+    v[0] = sum;
+    unrolled<1, H + 1>([&](auto J) {
+      constexpr int j = decltype(J)::value;
+      float2 m = a, s = make_float2(0.f, 0.f);
+      unrolled<1, H + 1>([&](auto K) {
+        constexpr int k = decltype(K)::value;
+        constexpr float c = Root<P, (j * k) % P>::re, sn = -Root<P, (j * k) % P>::im;
+        m = make_float2(m.x + c * t[k - 1].x, m.y + c * t[k - 1].y);
+        s = make_float2(s.x + sn * u[k - 1].x, s.y + sn * u[k - 1].y);
+      });
+      const float2 q = mul_mi(s);
+      v[j] = cadd(m, q);
+      v[P - j] = csub(m, q);
+    });
+  }
+};
+template <>
+struct Dft<7> : DftPrime<7> {};
+
+constexpr int gcd_of(int a, int b) { return b == 0 ? a : gcd_of(b, a % b); }
+constexpr int inverse_mod(int a, int m) {
+  for (int x = 1; x < m; ++x)
+    if (a * x % m == 1) return x;
+  return 1;
+}
+
+// N = A B.  Coprime: n = (B n1 + A n2) mod N, k = (B (1/B mod A) k1 +
+// A (1/A mod B) k2) mod N turns the DFT into A x B DFTs without twiddles.
+// Otherwise n = A n2 + n1, k = k1 + B k2: size-B DFTs over n2, twiddles
+// exp(-2 pi i n1 k1 / N), size-A DFTs over n1.
+template <int A, int B>
+struct DftPair {
+  TFFT_HD static void run(float2* v) {
+    constexpr int N = A * B;
+    constexpr bool coprime = gcd_of(A, B) == 1;
+    float2 y[A][B];
+    unrolled<0, A>([&](auto N1) {
+      constexpr int n1 = decltype(N1)::value;
+#pragma unroll
+      for (int n2 = 0; n2 < B; ++n2) y[n1][n2] = v[coprime ? (B * n1 + A * n2) % N : A * n2 + n1];
+      Dft<B>::run(y[n1]);
+      if constexpr (!coprime && n1 > 0)
+        unrolled<1, B>([&](auto K1) {
+          constexpr int k1 = decltype(K1)::value;
+          y[n1][k1] = cmul(y[n1][k1], make_float2(Root<N, n1 * k1>::re, Root<N, n1 * k1>::im));
+        });
+    });
+#pragma unroll
+    for (int k1 = 0; k1 < B; ++k1) {
+      float2 z[A];
+#pragma unroll
+      for (int n1 = 0; n1 < A; ++n1) z[n1] = y[n1][k1];
+      Dft<A>::run(z);
+#pragma unroll
+      for (int k2 = 0; k2 < A; ++k2)
+        v[coprime ? (A * inverse_mod(A % B, B) * k1 + B * inverse_mod(B % A, A) * k2) % N : k1 + B * k2] = z[k2];
+    }
+  }
+};
+template <>
+struct Dft<6> : DftPair<2, 3> {};
+template <>
+struct Dft<9> : DftPair<3, 3> {};
+template <>
+struct Dft<10> : DftPair<2, 5> {};
+template <>
+struct Dft<12> : DftPair<3, 4> {};
+template <>
+struct Dft<14> : DftPair<2, 7> {};
+template <>
+struct Dft<15> : DftPair<3, 5> {};
+template <>
+struct Dft<18> : DftPair<2, 9> {};
+template <>
+struct Dft<20> : DftPair<4, 5> {};
+template <>
+struct Dft<21> : DftPair<3, 7> {};
+template <>
+struct Dft<24> : DftPair<3, 8> {};
+template <>
+struct Dft<25> : DftPair<5, 5> {};
+template <>
+struct Dft<27> : DftPair<3, 9> {};
+template <>
+struct Dft<28> : DftPair<4, 7> {};
+template <>
+struct Dft<30> : DftPair<2, 15> {};
+
 // ------------------------------------------------------------ Stockham schedule
 //
 // A length-L FFT with radices R_0, R_1, ... (product L).  Stage s has span

@@ -329,6 +329,8 @@ bool kernel_supports_E(int E);
 // Compile-time specialised passes (tfft_spec.cu): the plan of length L if one
 // exists (and the buffers fit 32-bit offsets), and their launchers.
 bool spec_plan(int L, bool strided, int64_t nelems, AxisPlan& ap, int& width);
+// The plan of a real-line pass whose complex half-length is L, if compiled.
+bool real_plan(int L, int64_t nelems, AxisPlan& ap, int& width);
 cudaError_t launch_contig_spec(const ContigArgs& a, cudaStream_t s);
 cudaError_t launch_strided_spec(const StridedArgs& a, cudaStream_t s);
 cudaError_t launch_real_spec(const RealArgs& a, cudaStream_t s);

@@ -383,7 +383,7 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
       const int Lh = (int)(p->shape[ndims - 1] / 2);
       int width = 0;
       p->rplan = AxisPlan{};
-      if (spec_plan(Lh, false, p->nelems, p->rplan, width)) {
+      if (real_plan(Lh, p->nelems, p->rplan, width)) {
         p->rplan.width = width;
         if (!p->tw_off.count(Lh)) p->tw_off[Lh] = image_add(p, nullptr, (size_t)Lh * sizeof(float2));
         if (!p->tw_off.count(2 * Lh)) p->tw_off[2 * Lh] = image_add(p, nullptr, (size_t)2 * Lh * sizeof(float2));
@@ -396,6 +396,19 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
       const int L = (int)p->cshape[m];
       if (p->aplan.count(L)) continue;
       AxisPlan ap{}, aps{};
+      int wc = 0, ws = 0;
+      // lengths with a factor 7 that have compiled passes; the other lengths
+      // without a 2/3/5 factorisation go through Bluestein
+      const bool spec7 = !is_smooth_235(L) && spec_plan(L, false, p->nelems, ap, wc) &&
+                         spec_plan(L, true, p->nelems, aps, ws);
+      if (spec7) {
+        ap.width = wc;
+        aps.width = ws;
+        p->aplan[L] = ap;
+        p->aplan_s[L] = aps;
+        if (!p->tw_off.count(L)) p->tw_off[L] = image_add(p, nullptr, (size_t)L * sizeof(float2));
+        continue;
+      }
       if (!is_smooth_235(L) && L <= MAXLEN / 2) {
         if (!make_bluestein(p, L)) p->transformable = false;
         continue;

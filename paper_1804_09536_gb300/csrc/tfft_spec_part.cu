@@ -1,0 +1,32 @@
+// One part of the specialised passes: the rows L of tfft_spec_table.h with
+// L mod kSpecParts == TFFT_SPEC_PART (set by the build).
+#include "tfft_spec_pass.cuh"
+
+namespace tfft {
+namespace spec {
+
+template <int P>
+cudaError_t contig_part(const ContigArgs& a, cudaStream_t s) {
+#define X(LL, T, B, MB, ...)                  \
+  if constexpr (LL % kSpecParts == P)         \
+    if (a.ap.L == LL) return run_contig<LL, T, B, MB, __VA_ARGS__>(a, s);
+  TFFT_CONTIG_LINES(X)
+#undef X
+  return cudaErrorInvalidValue;
+}
+
+template <int P>
+cudaError_t strided_part(const StridedArgs& a, cudaStream_t s) {
+#define X(LL, T, W, MB, ...)                  \
+  if constexpr (LL % kSpecParts == P)         \
+    if (a.ap.L == LL) return run_strided<LL, T, W, MB, __VA_ARGS__>(a, s);
+  TFFT_STRIDED_LINES(X)
+#undef X
+  return cudaErrorInvalidValue;
+}
+
+template cudaError_t contig_part<TFFT_SPEC_PART>(const ContigArgs& a, cudaStream_t s);
+template cudaError_t strided_part<TFFT_SPEC_PART>(const StridedArgs& a, cudaStream_t s);
+
+}  // namespace spec
+}  // namespace tfft

@@ -1,0 +1,99 @@
+// Compile-time specialised FFT passes (contiguous and strided): the kernels
+// and launchers of the rows of tfft_spec_table.h.  Same Stockham schedule as
+// the runtime-dispatched kernels (tfft_kernels.cu), but with the length, the
+// radix sequence, the threads per line and the tile width fixed at compile
+// time: every index, span and twiddle stride folds to a constant, the row
+// tables hold 32-bit offsets, and the register budget is known to ptxas.
+#pragma once
+
+#include <type_traits>
+
+#include "tfft_internal.h"
+#include "tfft_spec_table.h"
+#include "tfft_tiles.cuh"
+
+namespace tfft {
+namespace spec {
+
+using namespace tiles;
+
+// Registers sized for MB resident CTAs (1024 threads per SM for plans of up
+// to 16 values per thread): more lines in flight per SM.  Against a
+// 512-thread target: 256^3 pass 49.4 -> 46.7 us, 128^4 0.667 -> 0.603 ms.
+template <int L, int T, int B, int MB, int... Rs>
+__global__ void __launch_bounds__(T * B, MB) k_contig_spec(const ContigArgs a) {
+  extern __shared__ float2 smem[];
+  for (int64_t tile = blockIdx.x; tile * B < a.nlines; tile += gridDim.x)
+    contig_tile<L, T, B, false, Rs...>(a, tile, smem, opaque_tid_x(), threadIdx.y);
+}
+
+// Whether the plain strided kernel keeps the rows' part/index table for the
+// CTA's lifetime (2L words): not at 4096, where it would halve the CTAs per SM.
+__host__ __device__ constexpr bool strided_cache_rows(int L) { return L <= 2048; }
+
+template <int L, int T, int W, int MB, int... Rs>
+__global__ void __launch_bounds__(W * T, MB) k_strided_spec(const StridedArgs a) {
+  extern __shared__ float2 smem[];
+  const int64_t ntiles = a.nouter * a.ncolblocks;
+  const int tid = threadIdx.y * W + threadIdx.x;
+  uint32_t* rp = nullptr;
+  if constexpr (strided_cache_rows(L)) {
+    rp = strided_rowparts<L, W>(smem);
+    strided_rowparts_init<L>(a, rp, tid, W * T);  // published by the first tile's barriers
+  }
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+    strided_tile<L, T, W, false, Rs...>(a, tile, smem, threadIdx.x, opaque_tid_y(), tid, rp);
+}
+
+// the kernel's shared-memory limit raised to 227 KB, once per device
+#define TFFT_ALLOW_SMEM(kernel)                          \
+  static PerDevice<cudaError_t> attr_cache;              \
+  const cudaError_t attr = smem_attr_once(attr_cache, kernel, 227 * 1024)
+
+constexpr int64_t kMaxGrid = 1 << 20;
+
+template <int L, int T, int B, int MB, int... Rs>
+cudaError_t run_contig(const ContigArgs& a, cudaStream_t s) {
+  TFFT_ALLOW_SMEM((k_contig_spec<L, T, B, MB, Rs...>));
+  if (attr != cudaSuccess) return attr;
+  const size_t smem = (size_t)B * line_pitch<L, Rs...>() * sizeof(float2);
+  int64_t grid = (a.nlines + B - 1) / B;
+  if (grid > kMaxGrid) grid = kMaxGrid;
+  if (grid < 1) return cudaSuccess;
+  k_contig_spec<L, T, B, MB, Rs...><<<(unsigned)grid, dim3(T, B), smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+template <int L, int T, int W, int MB, int... Rs>
+cudaError_t run_strided(const StridedArgs& a, cudaStream_t s) {
+  TFFT_ALLOW_SMEM((k_strided_spec<L, T, W, MB, Rs...>));
+  if (attr != cudaSuccess) return attr;
+  if (a.W != W) return cudaErrorInvalidValue;
+  constexpr size_t smem = strided_tile_smem<L, W>(strided_cache_rows(L));
+  // persistent: as many CTAs as fit at once, each taking every gridDim-th
+  // tile, so that the row part table is computed once per CTA
+  static PerDevice<int64_t> slots_cache;
+  const int64_t slots = slots_cache.get(current_device(), [] {
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_strided_spec<L, T, W, MB, Rs...>, W * T, smem);
+    return (int64_t)device_sm_count() * (per_sm > 0 ? per_sm : 1);
+  });
+  int64_t grid = a.nouter * a.ncolblocks;
+  if (grid > slots) grid = slots;
+  if (grid < 1) return cudaSuccess;
+  k_strided_spec<L, T, W, MB, Rs...><<<(unsigned)grid, dim3(W, T), smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+// The rows are compiled in kSpecParts translation units (tfft_spec_part.cu),
+// row L in part L mod kSpecParts (a prime above 7 spreads the 2/3/5/7 lengths
+// evenly).
+constexpr int kSpecParts = 11;
+
+template <int P>
+cudaError_t contig_part(const ContigArgs& a, cudaStream_t s);
+template <int P>
+cudaError_t strided_part(const StridedArgs& a, cudaStream_t s);
+
+}  // namespace spec
+}  // namespace tfft

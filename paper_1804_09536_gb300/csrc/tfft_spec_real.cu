@@ -22,10 +22,10 @@ using namespace tiles;
 // z = backward FFT_L(Z), x[2n] = Re z[n], x[2n+1] = Im z[n]; the imaginary
 // parts of X[0] and X[L] are ignored (taken as zero).
 
-template <int L, int E, int B, int... Rs>
-__global__ void __launch_bounds__((L / E) * B, min_blocks(E, (L / E) * B, 1024))
+template <int L, int T, int B, int MB, int... Rs>
+__global__ void __launch_bounds__(T * B, MB)
     k_r2c_spec(const RealArgs a) {
-  constexpr int T = L / E, NST = sizeof...(Rs);
+  constexpr int NST = sizeof...(Rs);
   constexpr int LP = line_pitch<L, Rs...>();
   constexpr int P = pad_every<Rs...>();
   extern __shared__ float2 smem[];
@@ -37,40 +37,40 @@ __global__ void __launch_bounds__((L / E) * B, min_blocks(E, (L / E) * B, 1024))
     const float2* src = reinterpret_cast<const float2*>(a.rin) + line * L;
     float2* dst = a.cout + line * a.cpitch;
     const int jt = opaque_tid_x();
-    float2 v[emax<L, E, Rs...>()];
+    float2 v[emax<L, T, Rs...>()];
     static_for<0, NST>([&](auto S) {
       constexpr int s = decltype(S)::value;
       constexpr int R = radix_at<s, Rs...>();
       constexpr int Ns = span_at<s, Rs...>();
       if constexpr (s == 0) {
 #pragma unroll
-        for (int q = 0; q < nbf<L, E, R>(); ++q)
+        for (int q = 0; q < nbf<L, T, R>(); ++q)
 #pragma unroll
           for (int r = 0; r < R; ++r)
-            v[q * R + r] = (act && bf_exists<L, E, R>(jt, q)) ? src[jt + q * T + r * (L / R)] : make_float2(0.f, 0.f);
+            v[q * R + r] = (act && bf_exists<L, T, R>(jt, q)) ? src[jt + q * T + r * (L / R)] : make_float2(0.f, 0.f);
       } else {
         constexpr int Rp = radix_at<s - 1, Rs...>();
         constexpr int Nsp = Ns / Rp;
         line_sync<T>();
 #pragma unroll
-        for (int q = 0; q < nbf<L, E, Rp>(); ++q)
-          if (bf_exists<L, E, Rp>(jt, q))
+        for (int q = 0; q < nbf<L, T, Rp>(); ++q)
+          if (bf_exists<L, T, Rp>(jt, q))
 #pragma unroll
             for (int r = 0; r < Rp; ++r) sl[padp<P>(stockham_out_index(jt + q * T, Nsp, Rp, r))] = v[q * Rp + r];
         line_sync<T>();
 #pragma unroll
-        for (int q = 0; q < nbf<L, E, R>(); ++q)
-          if (bf_exists<L, E, R>(jt, q))
+        for (int q = 0; q < nbf<L, T, R>(); ++q)
+          if (bf_exists<L, T, R>(jt, q))
 #pragma unroll
             for (int r = 0; r < R; ++r) v[q * R + r] = sl[padp<P>(jt + q * T + r * (L / R))];
       }
-      spec_stage<L, E, R, Ns>(v, jt, a.tw);
+      spec_stage<L, T, R, Ns>(v, jt, a.tw);
     });
     constexpr int RL = radix_at<NST - 1, Rs...>();
     line_sync<T>();
 #pragma unroll
-    for (int q = 0; q < nbf<L, E, RL>(); ++q)
-      if (bf_exists<L, E, RL>(jt, q))
+    for (int q = 0; q < nbf<L, T, RL>(); ++q)
+      if (bf_exists<L, T, RL>(jt, q))
 #pragma unroll
         for (int r = 0; r < RL; ++r) sl[padp<P>(jt + q * T + r * (L / RL))] = v[q * RL + r];
     line_sync<T>();
@@ -92,10 +92,10 @@ __global__ void __launch_bounds__((L / E) * B, min_blocks(E, (L / E) * B, 1024))
   }
 }
 
-template <int L, int E, int B, int... Rs>
-__global__ void __launch_bounds__((L / E) * B, min_blocks(E, (L / E) * B, 1024))
+template <int L, int T, int B, int MB, int... Rs>
+__global__ void __launch_bounds__(T * B, MB)
     k_c2r_spec(const RealArgs a) {
-  constexpr int T = L / E, NST = sizeof...(Rs);
+  constexpr int NST = sizeof...(Rs);
   constexpr int LP = line_pitch<L, Rs...>() + 1;
   constexpr int P = pad_every<Rs...>();
   extern __shared__ float2 smem[];
@@ -144,17 +144,17 @@ __global__ void __launch_bounds__((L / E) * B, min_blocks(E, (L / E) * B, 1024))
       }
     }
     line_sync<T>();
-    float2 v[emax<L, E, Rs...>()];
+    float2 v[emax<L, T, Rs...>()];
     static_for<0, NST>([&](auto S) {
       constexpr int s = decltype(S)::value;
       constexpr int R = radix_at<s, Rs...>();
       constexpr int Ns = span_at<s, Rs...>();
       if constexpr (s == 0) {
 #pragma unroll
-        for (int q = 0; q < nbf<L, E, R>(); ++q)
+        for (int q = 0; q < nbf<L, T, R>(); ++q)
 #pragma unroll
           for (int r = 0; r < R; ++r) {
-            const int k = bf_exists<L, E, R>(jt, q) ? jt + q * T + r * (L / R) : 0;
+            const int k = bf_exists<L, T, R>(jt, q) ? jt + q * T + r * (L / R) : 0;
             v[q * R + r] = sl[padp<P>(k)];
           }
       } else {
@@ -162,26 +162,26 @@ __global__ void __launch_bounds__((L / E) * B, min_blocks(E, (L / E) * B, 1024))
         constexpr int Nsp = Ns / Rp;
         line_sync<T>();
 #pragma unroll
-        for (int q = 0; q < nbf<L, E, Rp>(); ++q)
-          if (bf_exists<L, E, Rp>(jt, q))
+        for (int q = 0; q < nbf<L, T, Rp>(); ++q)
+          if (bf_exists<L, T, Rp>(jt, q))
 #pragma unroll
             for (int r = 0; r < Rp; ++r) sl[padp<P>(stockham_out_index(jt + q * T, Nsp, Rp, r))] = v[q * Rp + r];
         line_sync<T>();
 #pragma unroll
-        for (int q = 0; q < nbf<L, E, R>(); ++q)
-          if (bf_exists<L, E, R>(jt, q))
+        for (int q = 0; q < nbf<L, T, R>(); ++q)
+          if (bf_exists<L, T, R>(jt, q))
 #pragma unroll
             for (int r = 0; r < R; ++r) v[q * R + r] = sl[padp<P>(jt + q * T + r * (L / R))];
       }
-      spec_stage<L, E, R, Ns>(v, jt, a.tw);
+      spec_stage<L, T, R, Ns>(v, jt, a.tw);
     });
     constexpr int RL = radix_at<NST - 1, Rs...>();
 #pragma unroll
-    for (int q = 0; q < nbf<L, E, RL>(); ++q)
+    for (int q = 0; q < nbf<L, T, RL>(); ++q)
 #pragma unroll
       for (int r = 0; r < RL; ++r) {
         const float2 z = v[q * RL + r];
-        if (act && bf_exists<L, E, RL>(jt, q)) dst[jt + q * T + r * (L / RL)] = make_float2(z.x * a.scale, -z.y * a.scale);
+        if (act && bf_exists<L, T, RL>(jt, q)) dst[jt + q * T + r * (L / RL)] = make_float2(z.x * a.scale, -z.y * a.scale);
       }
   }
 }
@@ -193,37 +193,51 @@ __global__ void __launch_bounds__((L / E) * B, min_blocks(E, (L / E) * B, 1024))
 
 constexpr int64_t kMaxGrid = 1 << 20;
 
-template <int L, int E, int B, int... Rs>
+template <int L, int T, int B, int MB, int... Rs>
 cudaError_t run_real(const RealArgs& a, cudaStream_t s) {
   const int64_t grid0 = (a.nlines + B - 1) / B;
   const int64_t grid = grid0 > kMaxGrid ? kMaxGrid : grid0;
   if (grid < 1) return cudaSuccess;
   if (a.dir < 0) {
-    TFFT_ALLOW_SMEM((k_r2c_spec<L, E, B, Rs...>));
+    TFFT_ALLOW_SMEM((k_r2c_spec<L, T, B, MB, Rs...>));
     if (attr != cudaSuccess) return attr;
     const size_t smem = (size_t)B * line_pitch<L, Rs...>() * sizeof(float2);
-    k_r2c_spec<L, E, B, Rs...><<<(unsigned)grid, dim3(L / E, B), smem, s>>>(a);
+    k_r2c_spec<L, T, B, MB, Rs...><<<(unsigned)grid, dim3(T, B), smem, s>>>(a);
   } else {
-    TFFT_ALLOW_SMEM((k_c2r_spec<L, E, B, Rs...>));
+    TFFT_ALLOW_SMEM((k_c2r_spec<L, T, B, MB, Rs...>));
     if (attr != cudaSuccess) return attr;
     const size_t smem = (size_t)B * (line_pitch<L, Rs...>() + 1) * sizeof(float2);
-    k_c2r_spec<L, E, B, Rs...><<<(unsigned)grid, dim3(L / E, B), smem, s>>>(a);
+    k_c2r_spec<L, T, B, MB, Rs...><<<(unsigned)grid, dim3(T, B), smem, s>>>(a);
   }
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_real_spec(const RealArgs& a, cudaStream_t s) {
-  switch (a.ap.L) {
-#define X(L, EC, B, ES, W, ...) \
-  case L:                       \
-    return run_real<L, EC, B, __VA_ARGS__>(a, s);
-    TFFT_SPECS(X)
+namespace {
+
+constexpr bool real_length(int L) {
+#define X(LL) \
+  if (L == LL) return true;
+  TFFT_REAL_LENGTHS(X)
 #undef X
-    default:
-      return cudaErrorInvalidValue;
-  }
+  return false;
 }
+
+// the row of each real length (a template, so that the other rows are not
+// instantiated)
+template <class Args>
+cudaError_t launch_real_row(const Args& a, cudaStream_t s) {
+#define X(LL, T, B, MB, ...)                                              \
+  if constexpr (real_length(LL) && std::is_same<Args, RealArgs>::value) \
+    if (a.ap.L == LL) return run_real<LL, T, B, MB, __VA_ARGS__>(a, s);
+  TFFT_CONTIG_LINES(X)
+#undef X
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+cudaError_t launch_real_spec(const RealArgs& a, cudaStream_t s) { return launch_real_row(a, s); }
 
 }  // namespace tfft

@@ -34,47 +34,46 @@ __device__ __forceinline__ void static_for(F&& f) {
   }
 }
 
-// A line of length L has T = L / E threads.  A stage of radix R has L / R
+// A line of length L is worked by T threads.  A stage of radix R has L / R
 // butterflies, nbf = ceil((L / R) / T) per thread: butterfly j = jt + q T,
-// q < nbf, exists when j < L / R.  When every radix divides E this is E / R
-// butterflies each and no guard (the usual plans); lengths with 2, 3 and 5
-// all present (60, 120, 240, 480) have no such E, so their threads carry one
-// butterfly fewer in some stages and hold up to emax() values.
-template <int L, int E, int R>
+// q < nbf, exists when j < L / R.  When every radix divides L / T this is
+// L / (T R) butterflies each and no guard (the power-of-two plans); the
+// others guard, their threads carry one butterfly fewer in some stages and
+// hold up to emax() values.  T need not divide L.
+template <int L, int T, int R>
 __host__ __device__ constexpr int nbf() {
-  return (L / R + L / E - 1) / (L / E);
+  return (L / R + T - 1) / T;
 }
 
-template <int L, int E, int R>
+template <int L, int T, int R>
 __host__ __device__ constexpr bool nbf_exact() {
-  return (L / R) % (L / E) == 0;
+  return (L / R) % T == 0;
 }
 
-template <int L, int E, int... Rs>
+template <int L, int T, int... Rs>
 __host__ __device__ constexpr int emax() {
   constexpr int r[] = {Rs...};
   int m = 0;
   for (int i = 0; i < (int)sizeof...(Rs); ++i) {
-    const int v = ((L / r[i] + L / E - 1) / (L / E)) * r[i];
+    const int v = ((L / r[i] + T - 1) / T) * r[i];
     m = v > m ? v : m;
   }
   return m;
 }
 
 // Whether butterfly q of thread jt exists in a stage of radix R.
-template <int L, int E, int R>
+template <int L, int T, int R>
 __device__ __forceinline__ bool bf_exists(int jt, int q) {
-  if constexpr (nbf_exact<L, E, R>()) return true;
-  else return jt + q * (L / E) < L / R;
+  if constexpr (nbf_exact<L, T, R>()) return true;
+  else return jt + q * T < L / R;
 }
 
 // Twiddle (stage span Ns > 1) and size-R butterflies of a thread's work items.
-template <int L, int E, int R, int Ns, int EM>
+template <int L, int T, int R, int Ns, int EM>
 __device__ __forceinline__ void spec_stage(float2 (&v)[EM], int jt, const float2* __restrict__ tw) {
-  constexpr int T = L / E;
 #pragma unroll
-  for (int q = 0; q < nbf<L, E, R>(); ++q) {
-    if (!bf_exists<L, E, R>(jt, q)) continue;
+  for (int q = 0; q < nbf<L, T, R>(); ++q) {
+    if (!bf_exists<L, T, R>(jt, q)) continue;
     if constexpr (Ns > 1) {
       const int j = jt + q * T;
       const int step = (j % Ns) * (L / (Ns * R));
@@ -156,11 +155,11 @@ __host__ __device__ constexpr int min_blocks(int E, int threads, int target) {
   return t > 1 ? t : (E >= 20 && threads <= 256 ? 2 : 1);
 }
 
-// Synchronises the threads of one line: a warp (or part of one) when a line
-// has at most 32 threads, the whole CTA otherwise.
+// Synchronises the threads of one line: a warp when the line's threads lie
+// inside one (T divides 32), the whole CTA otherwise.
 template <int T>
 __device__ __forceinline__ void line_sync() {
-  if constexpr (T <= 32) {
+  if constexpr (32 % T == 0) {
     __syncwarp();
   } else {
     __syncthreads();
@@ -202,9 +201,9 @@ __device__ __forceinline__ float2 ld(const float2* p) {
 }
 
 // One group of B contiguous lines (group `tile`): thread jt of line ly.
-template <int L, int E, int B, bool CG, int... Rs>
+template <int L, int T, int B, bool CG, int... Rs>
 __device__ __forceinline__ void contig_tile(const ContigArgs& a, int64_t tile, float2* smem, int jt, int ly) {
-  constexpr int T = L / E, NST = sizeof...(Rs);
+  constexpr int NST = sizeof...(Rs);
   constexpr int LP = line_pitch<L, Rs...>();
   constexpr int P = pad_every<Rs...>();
   float2* sl = smem + ly * LP;
@@ -213,17 +212,17 @@ __device__ __forceinline__ void contig_tile(const ContigArgs& a, int64_t tile, f
   const bool act = line < a.nlines;
   const float2* src = a.in + line * L;
   float2* dst = a.out + line * L;
-  float2 v[emax<L, E, Rs...>()];
+  float2 v[emax<L, T, Rs...>()];
   static_for<0, NST>([&](auto S) {
     constexpr int s = decltype(S)::value;
     constexpr int R = radix_at<s, Rs...>();
     constexpr int Ns = span_at<s, Rs...>();
     if constexpr (s == 0) {
 #pragma unroll
-      for (int q = 0; q < nbf<L, E, R>(); ++q)
+      for (int q = 0; q < nbf<L, T, R>(); ++q)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-          float2 x = (act && bf_exists<L, E, R>(jt, q)) ? ld<CG>(src + jt + q * T + r * (L / R))
+          float2 x = (act && bf_exists<L, T, R>(jt, q)) ? ld<CG>(src + jt + q * T + r * (L / R))
                                                         : make_float2(0.f, 0.f);
           if (inv) x.y = -x.y;
           v[q * R + r] = x;
@@ -233,28 +232,28 @@ __device__ __forceinline__ void contig_tile(const ContigArgs& a, int64_t tile, f
       constexpr int Nsp = Ns / Rp;
       line_sync<T>();
 #pragma unroll
-      for (int q = 0; q < nbf<L, E, Rp>(); ++q)
-        if (bf_exists<L, E, Rp>(jt, q))
+      for (int q = 0; q < nbf<L, T, Rp>(); ++q)
+        if (bf_exists<L, T, Rp>(jt, q))
 #pragma unroll
           for (int r = 0; r < Rp; ++r) sl[padp<P>(stockham_out_index(jt + q * T, Nsp, Rp, r))] = v[q * Rp + r];
       line_sync<T>();
 #pragma unroll
-      for (int q = 0; q < nbf<L, E, R>(); ++q)
-        if (bf_exists<L, E, R>(jt, q))
+      for (int q = 0; q < nbf<L, T, R>(); ++q)
+        if (bf_exists<L, T, R>(jt, q))
 #pragma unroll
           for (int r = 0; r < R; ++r) v[q * R + r] = sl[padp<P>(jt + q * T + r * (L / R))];
     }
-    spec_stage<L, E, R, Ns>(v, jt, a.tw);
+    spec_stage<L, T, R, Ns>(v, jt, a.tw);
   });
   constexpr int RL = radix_at<NST - 1, Rs...>();
   const float oscale = contig_scale(a);
 #pragma unroll
-  for (int q = 0; q < nbf<L, E, RL>(); ++q)
+  for (int q = 0; q < nbf<L, T, RL>(); ++q)
 #pragma unroll
     for (int r = 0; r < RL; ++r) {
       float2 x = cscale(v[q * RL + r], oscale);
       if (inv) x.y = -x.y;
-      if (act && bf_exists<L, E, RL>(jt, q)) dst[jt + q * T + r * (L / RL)] = x;
+      if (act && bf_exists<L, T, RL>(jt, q)) dst[jt + q * T + r * (L / RL)] = x;
     }
   line_sync<T>();  // the line's shared slots are free for the next group
 }
@@ -326,10 +325,10 @@ __device__ __forceinline__ int row_offset(const DevLayout& lay, int axis, const 
 // column cx; tid = thread index in the CTA (W x T threads).  `rp` is the
 // per-CTA part/index table of strided_rowparts_init, or null (then each row
 // locates its part itself).
-template <int L, int E, int W, bool CG, int... Rs>
+template <int L, int T, int W, bool CG, int... Rs>
 __device__ __forceinline__ void strided_tile(const StridedArgs& a, int64_t tile, float2* smem, int cx, int jt,
                                              int tid, const uint32_t* rp = nullptr) {
-  constexpr int T = L / E, NST = sizeof...(Rs);
+  constexpr int NST = sizeof...(Rs);
   static_assert(W * T > 32, "the two layouts' folds are computed by threads 0 and 32");
   int* rin = reinterpret_cast<int*>(smem + L * W);
   int* rout = rin + L;
@@ -366,18 +365,18 @@ __device__ __forceinline__ void strided_tile(const StridedArgs& a, int64_t tile,
   __syncthreads();
   const int2 blk = ts->blk;
   const bool act = cx < blk.y;
-  float2 v[emax<L, E, Rs...>()];
+  float2 v[emax<L, T, Rs...>()];
   static_for<0, NST>([&](auto S) {
     constexpr int s = decltype(S)::value;
     constexpr int R = radix_at<s, Rs...>();
     constexpr int Ns = span_at<s, Rs...>();
     if constexpr (s == 0) {
 #pragma unroll
-      for (int q = 0; q < nbf<L, E, R>(); ++q)
+      for (int q = 0; q < nbf<L, T, R>(); ++q)
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const int pos = jt + q * T + r * (L / R);
-          float2 x = (act && bf_exists<L, E, R>(jt, q)) ? ld<CG>(a.in + rin[pos] + cx) : make_float2(0.f, 0.f);
+          float2 x = (act && bf_exists<L, T, R>(jt, q)) ? ld<CG>(a.in + rin[pos] + cx) : make_float2(0.f, 0.f);
           if (inv) x.y = -x.y;
           v[q * R + r] = x;
         }
@@ -386,28 +385,28 @@ __device__ __forceinline__ void strided_tile(const StridedArgs& a, int64_t tile,
       constexpr int Nsp = Ns / Rp;
       __syncthreads();
 #pragma unroll
-      for (int q = 0; q < nbf<L, E, Rp>(); ++q)
-        if (bf_exists<L, E, Rp>(jt, q))
+      for (int q = 0; q < nbf<L, T, Rp>(); ++q)
+        if (bf_exists<L, T, Rp>(jt, q))
 #pragma unroll
           for (int r = 0; r < Rp; ++r)
             smem[stockham_out_index(jt + q * T, Nsp, Rp, r) * W + cx] = v[q * Rp + r];
       __syncthreads();
 #pragma unroll
-      for (int q = 0; q < nbf<L, E, R>(); ++q)
-        if (bf_exists<L, E, R>(jt, q))
+      for (int q = 0; q < nbf<L, T, R>(); ++q)
+        if (bf_exists<L, T, R>(jt, q))
 #pragma unroll
           for (int r = 0; r < R; ++r) v[q * R + r] = smem[(jt + q * T + r * (L / R)) * W + cx];
     }
-    spec_stage<L, E, R, Ns>(v, jt, a.tw);
+    spec_stage<L, T, R, Ns>(v, jt, a.tw);
   });
   constexpr int RL = radix_at<NST - 1, Rs...>();
 #pragma unroll
-  for (int q = 0; q < nbf<L, E, RL>(); ++q)
+  for (int q = 0; q < nbf<L, T, RL>(); ++q)
 #pragma unroll
     for (int r = 0; r < RL; ++r) {
       float2 x = cscale(v[q * RL + r], a.scale);
       if (inv) x.y = -x.y;
-      if (act && bf_exists<L, E, RL>(jt, q)) a.out[rout[jt + q * T + r * (L / RL)] + cx] = x;
+      if (act && bf_exists<L, T, RL>(jt, q)) a.out[rout[jt + q * T + r * (L / RL)] + cx] = x;
     }
 }
 
@@ -422,10 +421,10 @@ __device__ __forceinline__ void strided_tile(const StridedArgs& a, int64_t tile,
 // jt + q T + r L / RL (natural order, self-sorting); between stages the
 // column goes through smem.  Starts and ends without a barrier: the caller
 // orders smem use around it.
-template <int L, int E, int W, int... Rs>
-__device__ __forceinline__ void strided_stages(float2 (&v)[emax<L, E, Rs...>()], float2* smem, int cx, int jt,
+template <int L, int T, int W, int... Rs>
+__device__ __forceinline__ void strided_stages(float2 (&v)[emax<L, T, Rs...>()], float2* smem, int cx, int jt,
                                                const float2* __restrict__ tw) {
-  constexpr int T = L / E, NST = sizeof...(Rs);
+  constexpr int NST = sizeof...(Rs);
   static_for<0, NST>([&](auto S) {
     constexpr int s = decltype(S)::value;
     constexpr int R = radix_at<s, Rs...>();
@@ -435,27 +434,27 @@ __device__ __forceinline__ void strided_stages(float2 (&v)[emax<L, E, Rs...>()],
       constexpr int Nsp = Ns / Rp;
       __syncthreads();
 #pragma unroll
-      for (int q = 0; q < nbf<L, E, Rp>(); ++q)
-        if (bf_exists<L, E, Rp>(jt, q))
+      for (int q = 0; q < nbf<L, T, Rp>(); ++q)
+        if (bf_exists<L, T, Rp>(jt, q))
 #pragma unroll
           for (int r = 0; r < Rp; ++r) smem[stockham_out_index(jt + q * T, Nsp, Rp, r) * W + cx] = v[q * Rp + r];
       __syncthreads();
 #pragma unroll
-      for (int q = 0; q < nbf<L, E, R>(); ++q)
-        if (bf_exists<L, E, R>(jt, q))
+      for (int q = 0; q < nbf<L, T, R>(); ++q)
+        if (bf_exists<L, T, R>(jt, q))
 #pragma unroll
           for (int r = 0; r < R; ++r) v[q * R + r] = smem[(jt + q * T + r * (L / R)) * W + cx];
     }
-    spec_stage<L, E, R, Ns>(v, jt, tw);
+    spec_stage<L, T, R, Ns>(v, jt, tw);
   });
 }
 
 // The same for one contiguous line in its padded line slot sl (the
 // contiguous passes' layout), synchronising the line's threads.
-template <int L, int E, int... Rs>
-__device__ __forceinline__ void line_stages(float2 (&v)[emax<L, E, Rs...>()], float2* sl, int jt,
+template <int L, int T, int... Rs>
+__device__ __forceinline__ void line_stages(float2 (&v)[emax<L, T, Rs...>()], float2* sl, int jt,
                                             const float2* __restrict__ tw) {
-  constexpr int T = L / E, NST = sizeof...(Rs);
+  constexpr int NST = sizeof...(Rs);
   constexpr int P = pad_every<Rs...>();
   static_for<0, NST>([&](auto S) {
     constexpr int s = decltype(S)::value;
@@ -466,18 +465,18 @@ __device__ __forceinline__ void line_stages(float2 (&v)[emax<L, E, Rs...>()], fl
       constexpr int Nsp = Ns / Rp;
       line_sync<T>();
 #pragma unroll
-      for (int q = 0; q < nbf<L, E, Rp>(); ++q)
-        if (bf_exists<L, E, Rp>(jt, q))
+      for (int q = 0; q < nbf<L, T, Rp>(); ++q)
+        if (bf_exists<L, T, Rp>(jt, q))
 #pragma unroll
           for (int r = 0; r < Rp; ++r) sl[padp<P>(stockham_out_index(jt + q * T, Nsp, Rp, r))] = v[q * Rp + r];
       line_sync<T>();
 #pragma unroll
-      for (int q = 0; q < nbf<L, E, R>(); ++q)
-        if (bf_exists<L, E, R>(jt, q))
+      for (int q = 0; q < nbf<L, T, R>(); ++q)
+        if (bf_exists<L, T, R>(jt, q))
 #pragma unroll
           for (int r = 0; r < R; ++r) v[q * R + r] = sl[padp<P>(jt + q * T + r * (L / R))];
     }
-    spec_stage<L, E, R, Ns>(v, jt, tw);
+    spec_stage<L, T, R, Ns>(v, jt, tw);
   });
 }
 
