@@ -26,32 +26,32 @@ using namespace tiles;
 using namespace tma;
 
 // Tile variants the executor can run, all with 256 threads per CTA:
-// id, kind (0 contiguous / 1 strided), length, elements per thread,
+// id, kind (0 contiguous / 1 strided), length, threads per line,
 // lines per group (contiguous) or tile width (strided), radices.
 #define TFFT_BATCH_VARIANTS(X)          \
   X(0, 0, 64, 8, 32, 8, 8)              \
-  X(1, 0, 96, 12, 32, 4, 4, 3, 2)       \
-  X(2, 0, 128, 16, 32, 16, 8)           \
-  X(3, 0, 160, 20, 32, 5, 4, 4, 2)      \
+  X(1, 0, 96, 8, 32, 16, 6)             \
+  X(2, 0, 128, 8, 32, 16, 8)            \
+  X(3, 0, 160, 16, 16, 16, 10)          \
   X(4, 0, 256, 16, 16, 16, 16)          \
-  X(5, 0, 256, 8, 8, 8, 8, 4)           \
-  X(6, 0, 128, 8, 16, 8, 8, 2)          \
-  X(7, 0, 32, 8, 64, 8, 4)              \
+  X(5, 0, 256, 32, 8, 8, 8, 4)          \
+  X(6, 0, 128, 16, 16, 8, 8, 2)         \
+  X(7, 0, 32, 4, 64, 8, 4)              \
   X(8, 1, 64, 8, 32, 8, 8)              \
-  X(9, 1, 96, 12, 32, 4, 4, 3, 2)       \
-  X(10, 1, 128, 16, 32, 16, 8)          \
-  X(11, 1, 160, 20, 32, 5, 4, 4, 2)     \
+  X(9, 1, 96, 8, 32, 8, 12)             \
+  X(10, 1, 128, 8, 32, 16, 8)           \
+  X(11, 1, 160, 16, 16, 16, 10)         \
   X(12, 1, 256, 16, 16, 16, 16)         \
-  X(13, 1, 256, 8, 8, 8, 8, 4)          \
-  X(14, 1, 128, 8, 16, 8, 8, 2)
+  X(13, 1, 256, 32, 8, 8, 8, 4)         \
+  X(14, 1, 128, 16, 16, 8, 8, 2)
 
-// TMA-staged strided variants: id, length, elements per thread, tile width
-// (W * L / E = 256 threads), radices.
+// TMA-staged strided variants: id, length, threads per column, tile width
+// (256 threads), radices.
 #define TFFT_BATCH_TMA_VARIANTS(X) \
   X(15, 64, 8, 32, 8, 8)           \
-  X(16, 128, 16, 32, 16, 8)        \
+  X(16, 128, 8, 32, 16, 8)         \
   X(17, 256, 16, 16, 16, 16)       \
-  X(18, 96, 12, 32, 4, 4, 3, 2)
+  X(18, 96, 8, 32, 8, 12)
 
 constexpr int kBatchThreads = 256;
 
@@ -70,10 +70,10 @@ __device__ __forceinline__ bool mbar_wait_cycles(uint64_t* bar, uint32_t parity,
 // ph[b] is the phase the next completion of buffer b's barrier will have
 // (the same in every thread).  Returns 0, or the device status bit of the
 // failure (TFFT_DEVICE_ETIMEOUT: a copy wait expired).
-template <int L, int E, int W, int... Rs>
+template <int L, int T, int W, int... Rs>
 __device__ int tma_item(const BatchSeg& S, int64_t t0, int64_t t1, float2* smem, int tid, uint64_t* bars,
                         uint32_t (&ph)[2], long long limit) {
-  constexpr int T = L / E, NST = sizeof...(Rs);
+  constexpr int NST = sizeof...(Rs);
   const StridedArgs& a = S.sa;
   const CUtensorMap* tin = static_cast<const CUtensorMap*>(S.tin);
   const CUtensorMap* tout = static_cast<const CUtensorMap*>(S.tout);
@@ -118,14 +118,15 @@ __device__ int tma_item(const BatchSeg& S, int64_t t0, int64_t t1, float2* smem,
       err = TFFT_DEVICE_ETIMEOUT;
       break;
     }
-    float2 v[E];
+    float2 v[emax<L, T, Rs...>()];
     static_for<0, NST>([&](auto St) {
       constexpr int s = decltype(St)::value;
       constexpr int R = radix_at<s, Rs...>();
       constexpr int Ns = span_at<s, Rs...>();
       if constexpr (s == 0) {
 #pragma unroll
-        for (int q = 0; q < E / R; ++q)
+        for (int q = 0; q < nbf<L, T, R>(); ++q)
+          if (bf_exists<L, T, R>(jt, q))
 #pragma unroll
           for (int r = 0; r < R; ++r) {
             float2 x = cur[(jt + q * T + r * (L / R)) * W + cx];
@@ -137,12 +138,14 @@ __device__ int tma_item(const BatchSeg& S, int64_t t0, int64_t t1, float2* smem,
         constexpr int Nsp = Ns / Rp;
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < E / Rp; ++q)
+        for (int q = 0; q < nbf<L, T, Rp>(); ++q)
+          if (bf_exists<L, T, Rp>(jt, q))
 #pragma unroll
           for (int r = 0; r < Rp; ++r) cur[stockham_out_index(jt + q * T, Nsp, Rp, r) * W + cx] = v[q * Rp + r];
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < E / R; ++q)
+        for (int q = 0; q < nbf<L, T, R>(); ++q)
+          if (bf_exists<L, T, R>(jt, q))
 #pragma unroll
           for (int r = 0; r < R; ++r) v[q * R + r] = cur[(jt + q * T + r * (L / R)) * W + cx];
       }
@@ -151,7 +154,8 @@ __device__ int tma_item(const BatchSeg& S, int64_t t0, int64_t t1, float2* smem,
     constexpr int RL = radix_at<NST - 1, Rs...>();
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < E / RL; ++q)
+    for (int q = 0; q < nbf<L, T, RL>(); ++q)
+          if (bf_exists<L, T, RL>(jt, q))
 #pragma unroll
       for (int r = 0; r < RL; ++r) {
         float2 x = cscale(v[q * RL + r], a.scale);
@@ -176,12 +180,12 @@ __device__ int tma_item(const BatchSeg& S, int64_t t0, int64_t t1, float2* smem,
   return err;
 }
 
-template <int KIND, int L, int E, int BW, int... Rs>
+template <int KIND, int L, int T, int BW, int... Rs>
 __device__ __forceinline__ void run_tile(const BatchSeg& S, int64_t tile, float2* smem, int tid) {
   if constexpr (KIND == 0)
-    contig_tile<L, L / E, BW, true, Rs...>(S.ca, tile, smem, tid % (L / E), tid / (L / E));
+    contig_tile<L, T, BW, true, Rs...>(S.ca, tile, smem, tid % T, tid / T);
   else
-    strided_tile<L, L / E, BW, true, Rs...>(S.sa, tile, smem, tid % BW, tid / BW, tid);
+    strided_tile<L, T, BW, true, false, Rs...>(S.sa, tile, smem, tid % BW, tid / BW, tid);
 }
 
 // Segments whose first-item table fits shared memory use it for the lookup.
@@ -274,9 +278,9 @@ __global__ void __launch_bounds__(kBatchThreads, 3) k_batch(const BatchArgs b) {
       // the tensor copies need a 128-byte aligned shared-memory end
       int err = (static_cast<uint32_t>(__cvta_generic_to_shared(smem)) & 127) ? TFFT_DEVICE_EALIGN : 0;
       if (!err) switch (S.variant) {
-#define X(ID, L, E, W, ...)                                                            \
+#define X(ID, L, T, W, ...)                                                            \
   case ID:                                                                             \
-    err = tma_item<L, E, W, __VA_ARGS__>(S, t0, t1, smem, tid, s_bars, ph, b.spin_limit); \
+    err = tma_item<L, T, W, __VA_ARGS__>(S, t0, t1, smem, tid, s_bars, ph, b.spin_limit); \
     break;
           TFFT_BATCH_TMA_VARIANTS(X)
 #undef X
@@ -294,9 +298,9 @@ __global__ void __launch_bounds__(kBatchThreads, 3) k_batch(const BatchArgs b) {
     } else
     for (int64_t tile = t0; tile < t1; ++tile) {
       switch (S.variant) {
-#define X(ID, KIND, L, E, BW, ...)                              \
+#define X(ID, KIND, L, T, BW, ...)                              \
   case ID:                                                      \
-    run_tile<KIND, L, E, BW, __VA_ARGS__>(S, tile, smem, tid);  \
+    run_tile<KIND, L, T, BW, __VA_ARGS__>(S, tile, smem, tid);  \
     break;
         TFFT_BATCH_VARIANTS(X)
 #undef X
@@ -313,7 +317,7 @@ __global__ void __launch_bounds__(kBatchThreads, 3) k_batch(const BatchArgs b) {
 
 constexpr size_t batch_smem() {
   size_t m = 0;
-#define X(ID, KIND, L, E, BW, ...)                                                                     \
+#define X(ID, KIND, L, T, BW, ...)                                                                     \
   {                                                                                                    \
     const size_t v = (KIND == 0) ? (size_t)BW * line_pitch<L, __VA_ARGS__>() * sizeof(float2) \
                                  : strided_tile_smem<L, BW>(false);                                 \
@@ -321,7 +325,7 @@ constexpr size_t batch_smem() {
   }
   TFFT_BATCH_VARIANTS(X)
 #undef X
-#define X(ID, L, E, W, ...)                                   \
+#define X(ID, L, T, W, ...)                                   \
   {                                                           \
     const size_t v = 2 * (size_t)L * W * sizeof(float2);      \
     m = v > m ? v : m;                                        \
@@ -335,17 +339,17 @@ constexpr size_t batch_smem() {
 
 bool batch_variant(int id, int& kind, int& L, int& E, int& BW, AxisPlan& ap) {
   switch (id) {
-#define X(ID, KIND, LL, EE, BWW, ...)                                   \
+#define X(ID, KIND, LL, TT, BWW, ...)                                   \
   case ID: {                                                            \
     const int r[] = {__VA_ARGS__};                                      \
     kind = KIND;                                                        \
     L = LL;                                                             \
-    E = EE;                                                             \
+    E = LL / TT;                                                          \
     BW = BWW;                                                           \
     ap = AxisPlan{};                                                    \
     ap.L = LL;                                                          \
-    ap.E = EE;                                                          \
-    ap.T = LL / EE;                                                     \
+    ap.E = LL / TT;                                                       \
+    ap.T = TT;                                                          \
     ap.nst = (int)(sizeof(r) / sizeof(int));                            \
     for (int s = 0; s < ap.nst; ++s) {                                  \
       ap.radix[s] = r[s];                                               \
@@ -357,17 +361,17 @@ bool batch_variant(int id, int& kind, int& L, int& E, int& BW, AxisPlan& ap) {
   }
     TFFT_BATCH_VARIANTS(X)
 #undef X
-#define X(ID, LL, EE, WW, ...)                                          \
+#define X(ID, LL, TT, WW, ...)                                          \
   case ID: {                                                            \
     const int r[] = {__VA_ARGS__};                                      \
     kind = 1;                                                           \
     L = LL;                                                             \
-    E = EE;                                                             \
+    E = LL / TT;                                                          \
     BW = WW;                                                            \
     ap = AxisPlan{};                                                    \
     ap.L = LL;                                                          \
-    ap.E = EE;                                                          \
-    ap.T = LL / EE;                                                     \
+    ap.E = LL / TT;                                                       \
+    ap.T = TT;                                                          \
     ap.nst = (int)(sizeof(r) / sizeof(int));                            \
     for (int s = 0; s < ap.nst; ++s) {                                  \
       ap.radix[s] = r[s];                                               \

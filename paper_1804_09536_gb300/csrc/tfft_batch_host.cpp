@@ -269,8 +269,8 @@ int batch_launch_streams(tfft_batch b, cudaStream_t st) {
     for (int t : b->lanes[j]) {
       if (rc) break;
       void* bufs[4] = {b->ins[t], b->outs[t], b->works[t], nullptr};
-      for (const Step& s : b->steps[t])
-        if ((rc = launch_step(b->plans[t], s, bufs, x))) break;
+      for (size_t k = 0; k < b->steps[t].size() && !rc; ++k)
+        rc = launch_step(b->plans[t], b->steps[t][k], bufs, x, chain_flags(b->plans[t], k) & ~kChainCarve);
     }
     cudaError_t e2 = cudaEventRecord(b->fork.done[j], x);
     if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(st, b->fork.done[j], 0);

@@ -39,6 +39,8 @@ __global__ void __launch_bounds__((M / E) * B, min_blocks(E, (M / E) * B, 512))
   const int ly = threadIdx.y;
   float2* sl = smem + ly * LP;
   const bool inv = a.sign > 0;
+  chain_next();
+  chain_wait();
   const float oscale = contig_scale(a);
   for (int64_t base = (int64_t)blockIdx.x * B; base < a.nlines; base += (int64_t)gridDim.x * B) {
     const int64_t line = base + ly;
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(W * (M / E), min_blocks(E, W * (M / E), 768))
   const int tid = threadIdx.y * W + cx;
   const bool inv = a.sign > 0;
   const int64_t ntiles = a.nouter * a.ncolblocks;
+  chain_next();
   // part and index of every row of both layouts, once per CTA
   for (int i = tid; i < 2 * N; i += W * T) {
     const bool out = i >= N;
@@ -156,6 +159,7 @@ __global__ void __launch_bounds__(W * (M / E), min_blocks(E, W * (M / E), 768))
     const int2 blk = ts->blk;
     const bool act = cx < blk.y;
     const int jt = opaque_tid_y();
+    if (tile == blockIdx.x) chain_wait();
     float2 v[E];
 #pragma unroll
     for (int q = 0; q < E / R0; ++q)
@@ -238,8 +242,7 @@ cudaError_t run_blue_contig(const ContigArgs& a, const BlueArgs& b, cudaStream_t
   int64_t grid = (a.nlines + B - 1) / B;
   if (grid > kMaxGrid) grid = kMaxGrid;
   if (grid < 1) return cudaSuccess;
-  k_blue_contig_spec<M, E, B, Rs...><<<(unsigned)grid, dim3(M / E, B), smem, s>>>(a, b);
-  return cudaGetLastError();
+  return launch_chained(k_blue_contig_spec<M, E, B, Rs...>, dim3((unsigned)grid), dim3(M / E, B), smem, s, a.chained, a, b);
 }
 
 template <int M, int E, int W, int... Rs>
@@ -259,8 +262,7 @@ cudaError_t run_blue_strided(const StridedArgs& a, const BlueArgs& b, cudaStream
   int64_t grid = a.nouter * a.ncolblocks;
   if (grid > slots) grid = slots;
   if (grid < 1) return cudaSuccess;
-  k_blue_strided_spec<M, E, W, Rs...><<<(unsigned)grid, dim3(W, M / E), smem, s>>>(a, b);
-  return cudaGetLastError();
+  return launch_chained(k_blue_strided_spec<M, E, W, Rs...>, dim3((unsigned)grid), dim3(W, M / E), smem, s, a.chained, a, b);
 }
 
 }  // namespace

@@ -26,12 +26,16 @@ Step fft_step(tfft_plan p, int axis, int lin, int lout, int sign) {
     auto cb = get_colblocks(p, lin, lout, s.W);
     s.cb_off = cb.first;
     s.ncb = cb.second;
-    int Et = 0, Wt = 0, wantE = 0;
-    const int wantW = tuned_width(s.L, &wantE);
-    s.tma = p->use_tma && ap.spec && tma_strided_variant(s.L, wantW, wantE, Et, Wt) &&
-            tma_geo(p, lin, axis, Wt, s.gin) && tma_geo(p, lout, axis, Wt, s.gout);
+    int Tt = 0, Wt = 0, wantT = 0;
+    const int wantW = tuned_width(s.L, &wantT);
+    auto geo = [&] { return tma_geo(p, lin, axis, Wt, s.gin) && tma_geo(p, lout, axis, Wt, s.gout); };
+    if (p->use_tma && ap.spec && wantW > 0) {
+      s.tma = tma_strided_variant(s.L, wantW, wantT, Tt, Wt) && geo();
+    } else if (p->use_tma && ap.spec) {
+      for (int k = 0; !s.tma && tma_strided_row(s.L, k, Tt, Wt); ++k) s.tma = geo();
+    }
     if (s.tma) {
-      s.tma_E = Et;
+      s.tma_T = Tt;
       s.tma_W = Wt;
       auto cbt = get_colblocks(p, lin, lout, Wt);
       s.tma_cb_off = cbt.first;
@@ -46,9 +50,9 @@ Step fft_step(tfft_plan p, int axis, int lin, int lout, int sign) {
     // uneven blocks: an in-place pass along axis 0 can still run TMA-staged
     // tiles over the layout's rank groups
     if (!s.tma && p->use_tma && ap.spec && lin == lout && axis == 0 &&
-        tma_strided_variant(s.L, wantW, wantE, Et, Wt) && rank_groups(p, lin, s.L, Wt, s.rg, s.rgh)) {
+        tma_strided_variant(s.L, wantW, wantT, Tt, Wt) && rank_groups(p, lin, s.L, Wt, s.rg, s.rgh)) {
       s.tma_groups = true;
-      s.tma_E = Et;
+      s.tma_T = Tt;
       s.tma_W = Wt;
     }
     // tensor-core plans: the tensor-core TMA variant of this length, with its
@@ -99,7 +103,7 @@ void add_window_pass(tfft_plan p, std::vector<Step>& v, int axis, int lin, int l
   };
   Step w = s;
   w.tma_win = true;
-  w.tma_E = p->win_E;
+  w.tma_T = p->win_T;
   w.tma_W = p->win_W;
   w.win_c0 = c0;
   w.win_nc = p->win_nc;
@@ -235,7 +239,23 @@ void assign_buffers(std::vector<Step>& v, bool destroy_input) {
   }
 }
 
-int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st) {
+// How pass k of a plan's step list is launched.  The passes of one call are
+// chained while a stage buffer has at most 32 MiB: a kernel then runs for a
+// few microseconds and its start-up is a good part of that (us per forward +
+// inverse, unchained / chained: 32^3 16.5 / 12.0, 60 x 72 x 100 29.3 / 26.8,
+// 100 x 150 x 180 72.5 / 70.5, 160^3 84.2 / 79.0).  Above, the waiting CTAs
+// take residency from the running pass (180 x 200 x 240 171 / 181, 256^3 266
+// / 274).  Up to 4 MiB every pass also takes the same carve-out (60 x 72 x
+// 100 24.4, 64^3 on 2 x 4 18.9 / 15.8 / 14.4); larger arrays want the L1
+// (100 x 150 x 180 71.7, 42 x 127 x 256 58.1 without and 60.6 with it).
+// The first pass starts after everything the caller queued before it.
+int chain_flags(tfft_plan p, size_t k) {
+  const int64_t bytes = p->nelems * (int64_t)sizeof(float2);
+  if (bytes > (int64_t(32) << 20)) return 0;
+  return (k > 0 ? kChainAfter : kChainFirst) | (bytes <= (int64_t(4) << 20) ? kChainCarve : 0);
+}
+
+int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st, int chained) {
   const float2* in = static_cast<const float2*>(bufs[s.src]) + s.in_shift;
   float2* out = static_cast<float2*>(bufs[s.dst]) + s.out_shift;
   cudaError_t e = cudaSuccess;
@@ -250,6 +270,7 @@ int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st) 
     a.sign = s.sign;
     a.scale = s.scaled ? (float)s.scale_value : 1.0f;
     a.coef = s.coef;
+    a.chained = chained;
     a.status = reinterpret_cast<int*>(p->d_state);
     a.wait_limit = p->wait_limit;
     if (a.ap.blue_m)
@@ -287,6 +308,7 @@ int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st) 
     a.scale = s.scaled ? (float)s.scale_value : 1.0f;
     a.status = reinterpret_cast<int*>(p->d_state);
     a.wait_limit = p->wait_limit;
+    a.chained = chained;
     bool done = false;
     if (s.tma_win) {
       alignas(64) CUtensorMap ti, to;
@@ -297,7 +319,7 @@ int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st) 
       at.colblocks = reinterpret_cast<const int2*>(p->d_state + s.tma_cb_off);
       at.ncolblocks = s.tma_ncb;
       at.outer_fastest = s.tma_outer_fastest ? 1 : 0;
-      e = launch_strided_tma(at, s.tma_E, s.gin, s.gout, &ti, &to, st);
+      e = launch_strided_tma(at, s.tma_T, s.gin, s.gout, &ti, &to, st);
       done = true;
     }
     if (!done && s.tc) {
@@ -322,7 +344,7 @@ int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st) 
         at.colblocks = reinterpret_cast<const int2*>(p->d_state + s.tma_cb_off);
         at.ncolblocks = s.tma_ncb;
         at.outer_fastest = s.tma_outer_fastest ? 1 : 0;
-        e = launch_strided_tma(at, s.tma_E, s.gin, s.gout, &ti, &to, st);
+        e = launch_strided_tma(at, s.tma_T, s.gin, s.gout, &ti, &to, st);
         done = true;
       }
     }
@@ -339,7 +361,7 @@ int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st) 
       if (ok) {
         StridedArgs at = a;
         at.W = s.tma_W;
-        e = launch_strided_tma_groups(at, s.tma_E, s.rg, pin, pout, st);
+        e = launch_strided_tma_groups(at, s.tma_T, s.rg, pin, pout, st);
         done = true;
       }
     }
@@ -360,6 +382,7 @@ int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st) 
     a.tw = reinterpret_cast<const float2*>(p->d_state + p->tw_off[p->rplan.L]);
     a.tw2 = reinterpret_cast<const float2*>(p->d_state + p->tw_off[2 * p->rplan.L]);
     a.dir = s.sign;
+    a.chained = chained;
     a.scale = s.scaled ? (float)s.scale_value : 1.0f;
     a.status = reinterpret_cast<int*>(p->d_state);
     e = launch_real_spec(a, st);
@@ -383,7 +406,7 @@ int run_steps(tfft_plan p, const std::vector<Step>& steps, void* const* bufs, cu
       cudaError_t e = cudaEventRecord(p->events[k], st);
       if (e != cudaSuccess) return cuda_fail(e, "cudaEventRecord");
     }
-    int rc = launch_step(p, steps[k], bufs, st);
+    int rc = launch_step(p, steps[k], bufs, st, timed ? 0 : chain_flags(p, k));
     if (rc != TFFT_OK) return rc;
   }
   if (timed) {

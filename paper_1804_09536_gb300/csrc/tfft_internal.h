@@ -16,6 +16,17 @@ constexpr int TFFT_DEVICE_ETIMEOUT = 1;  // a bounded wait on a copy expired
 constexpr int TFFT_DEVICE_EALIGN = 2;    // a TMA tile buffer was not 128-byte aligned (copy skipped)
 constexpr int TFFT_DEVICE_ETMEM = 4;     // MMAs still running after the clean-up wait: tensor memory not released
 
+// How a pass is launched in a chain of passes (launch_chained()).
+constexpr int kChainAfter = 1;  // may start before the previous kernel has finished
+constexpr int kChainFirst = 4;  // the first pass of a chain: the next may start before it has finished
+constexpr int kChainCarve = 2;  // largest shared-memory carve-out, the same for the whole chain
+
+// Lengths whose passes have a chained variant beside the plain one, which is
+// compiled without the chain instructions: in the large passes, which are
+// never chained, those cost 0.3-1.2 % (512^3 1946 -> 1971 us, 128^4 5312 ->
+// 5331).
+constexpr bool chainable(int L) { return L <= 256; }
+
 // Batched 1-D FFT of contiguous lines (the axis held whole and innermost,
 // Eq. pencil0 / slab0): line l of the buffer is elements [l L, (l + 1) L).
 struct ContigArgs {
@@ -30,6 +41,7 @@ struct ContigArgs {
   const double* coef;   // optional device factor on the output (NULL: none)
   int* status;       // device status word
   uint32_t wait_limit;  // polls of a bounded copy wait (TMA passes)
+  int chained;       // kChain* bits, see launch_chained
 };
 
 // Bluestein's algorithm for a line length N without a 2/3/5 factorisation:
@@ -44,6 +56,41 @@ struct BlueArgs {
 };
 
 #ifdef __CUDACC__
+// A pass launched as a programmatic dependent of the kernel before it in the
+// stream (kChainAfter): its CTAs may start while that kernel drains, so
+// everything up to chain_wait() -- index tables, twiddles, barriers --
+// overlaps it.  A kernel launched this way reads and writes no array before
+// chain_wait(), which returns once the previous kernel has completed and its
+// stores are visible; chain_next() lets the kernel after it start.  Both do
+// nothing in a launch without the attribute.  CTAs of two kernels share an SM
+// only under one shared-memory / L1 split, so the passes of the smallest
+// plans all ask for the largest shared memory (kChainCarve).
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int chained,
+                           const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2] = {};
+  int n = 0;
+  if (chained & kChainCarve) {
+    attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[n++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+  }
+  if (chained & kChainAfter) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Output factor of a contiguous pass: the host's scale, times the device
 // coefficient when there is one (formed in double, applied in float).
 __device__ __forceinline__ float contig_scale(const ContigArgs& a) {
@@ -67,6 +114,7 @@ struct RealArgs {
   int dir;
   float scale;
   int* status;
+  int chained;          // kChain* bits, see launch_chained
 };
 
 // 1-D FFT along axis `axis` < d - 1 with the redistribution fused into the
@@ -95,6 +143,7 @@ struct StridedArgs {
   float scale;
   int* status;            // device status word
   uint32_t wait_limit;    // polls of a bounded copy wait (TMA passes)
+  int chained;            // kChain* bits, see launch_chained
 };
 
 #ifdef __CUDACC__
@@ -336,14 +385,16 @@ cudaError_t launch_strided_spec(const StridedArgs& a, cudaStream_t s);
 cudaError_t launch_real_spec(const RealArgs& a, cudaStream_t s);
 
 // TMA-staged passes (tfft_tma.cu).  tmap_* point to host CUtensorMap objects.
-// tma_strided_variant: elements per thread and tile width of the strided TMA
+// tma_strided_variant: threads per column and tile width of the strided TMA
 // variant of length L with width want_W if compiled, else the default one.
-bool tma_strided_variant(int L, int want_W, int want_E, int& E, int& W);
-cudaError_t launch_strided_tma(const StridedArgs& a, int E, const TmaGeo& gin, const TmaGeo& gout,
+bool tma_strided_variant(int L, int want_W, int want_T, int& T, int& W);
+// Row k of the variants of length L (false past the last).
+bool tma_strided_row(int L, int k, int& T, int& W);
+cudaError_t launch_strided_tma(const StridedArgs& a, int T, const TmaGeo& gin, const TmaGeo& gout,
                                const void* tmap_in, const void* tmap_out, cudaStream_t s);
 // The same passes over the rank groups of an uneven layout (in place along
 // the leading axis): tmaps_in / tmaps_out hold g.ngroups host CUtensorMaps each.
-cudaError_t launch_strided_tma_groups(const StridedArgs& a, int E, const RankGroupGeo& g, const void* const* tmaps_in,
+cudaError_t launch_strided_tma_groups(const StridedArgs& a, int T, const RankGroupGeo& g, const void* const* tmaps_in,
                                       const void* const* tmaps_out, cudaStream_t s);
 
 }  // namespace tfft

@@ -97,7 +97,7 @@ struct Step {
   // TMA-staged strided pass: variant, its column blocks and the tile
   // geometry of the input and output layouts
   bool tma = false;
-  int tma_E = 0, tma_W = 0;
+  int tma_T = 0, tma_W = 0;
   size_t tma_cb_off = 0;
   int64_t tma_ncb = 0;
   bool tma_outer_fastest = false;  // tile order of the TMA pass
@@ -170,7 +170,7 @@ struct tfft_plan_s {
   int pad_stage = -1;
   int64_t pad_lead = 0;
   int64_t win_c0 = 0, win_nc = 0;  // the TMA column window of that pass
-  int win_E = 0, win_W = 0;        // its TMA variant
+  int win_T = 0, win_W = 0;        // its TMA variant
   uint32_t wait_limit = 1u << 22;  // polls of a bounded copy wait
   std::vector<LayoutH> st;
   std::map<int, AxisPlan> aplan;   // contiguous-line passes
@@ -281,7 +281,7 @@ Step box_step(const BoxList& L);
 int split_rows(int L);
 bool tma_geo(tfft_plan p, int stage, int axis, int W, TmaGeo& G);
 bool encode_stage_map(tfft_plan p, const TmaGeo& G, int axis, int W, const void* base, CUtensorMap* map);
-int tuned_width(int L, int* E = nullptr, const char* var = "TFFT_TMA_W");
+int tuned_width(int L, int* T = nullptr, const char* var = "TFFT_TMA_W");
 bool rank_groups(tfft_plan p, int stage, int L, int W, RankGroupGeo& G, std::vector<RankGroupH>& groups);
 bool encode_group_map(const RankGroupH& H, int L, int W, const void* base, CUtensorMap* map);
 bool window_side(tfft_plan p, int stage, int axis, int W, int64_t c0, int64_t nc, int64_t shift, TmaGeo& G,
@@ -295,7 +295,8 @@ Step fft_step(tfft_plan p, int axis, int lin, int lout, int sign);
 Step last_axis_step(tfft_plan p, int sign);
 std::vector<Step> build_steps(tfft_plan p, int sign, int mode);
 void assign_buffers(std::vector<Step>& v, bool destroy_input);
-int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st);
+int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st, int chained = 0);
+int chain_flags(tfft_plan p, size_t k);
 int run_steps(tfft_plan p, const std::vector<Step>& steps, void* const* bufs, cudaStream_t st);
 int run_steps_cached(tfft_plan p, const tfft_plan_s::GraphKey& k, const std::vector<Step>& steps, void* const* bufs,
                      cudaStream_t st);

@@ -9,7 +9,7 @@ template <int P>
 cudaError_t contig_part(const ContigArgs& a, cudaStream_t s) {
 #define X(LL, T, B, MB, ...)                  \
   if constexpr (LL % kSpecParts == P)         \
-    if (a.ap.L == LL) return run_contig<LL, T, B, MB, __VA_ARGS__>(a, s);
+    if (a.ap.L == LL) return run_contig<LL, T, B, MB, false, __VA_ARGS__>(a, s);
   TFFT_CONTIG_LINES(X)
 #undef X
   return cudaErrorInvalidValue;
@@ -19,7 +19,7 @@ template <int P>
 cudaError_t strided_part(const StridedArgs& a, cudaStream_t s) {
 #define X(LL, T, W, MB, ...)                  \
   if constexpr (LL % kSpecParts == P)         \
-    if (a.ap.L == LL) return run_strided<LL, T, W, MB, __VA_ARGS__>(a, s);
+    if (a.ap.L == LL) return run_strided<LL, T, W, MB, false, __VA_ARGS__>(a, s);
   TFFT_STRIDED_LINES(X)
 #undef X
   return cudaErrorInvalidValue;

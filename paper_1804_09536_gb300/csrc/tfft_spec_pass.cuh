@@ -20,9 +20,13 @@ using namespace tiles;
 // Registers sized for MB resident CTAs (1024 threads per SM for plans of up
 // to 16 values per thread): more lines in flight per SM.  Against a
 // 512-thread target: 256^3 pass 49.4 -> 46.7 us, 128^4 0.667 -> 0.603 ms.
-template <int L, int T, int B, int MB, int... Rs>
+template <int L, int T, int B, int MB, bool CHAIN, int... Rs>
 __global__ void __launch_bounds__(T * B, MB) k_contig_spec(const ContigArgs a) {
   extern __shared__ float2 smem[];
+  if constexpr (CHAIN) {
+    chain_next();
+    chain_wait();
+  }
   for (int64_t tile = blockIdx.x; tile * B < a.nlines; tile += gridDim.x)
     contig_tile<L, T, B, false, Rs...>(a, tile, smem, opaque_tid_x(), threadIdx.y);
 }
@@ -31,18 +35,19 @@ __global__ void __launch_bounds__(T * B, MB) k_contig_spec(const ContigArgs a) {
 // CTA's lifetime (2L words): not at 4096, where it would halve the CTAs per SM.
 __host__ __device__ constexpr bool strided_cache_rows(int L) { return L <= 2048; }
 
-template <int L, int T, int W, int MB, int... Rs>
+template <int L, int T, int W, int MB, bool CHAIN, int... Rs>
 __global__ void __launch_bounds__(W * T, MB) k_strided_spec(const StridedArgs a) {
   extern __shared__ float2 smem[];
   const int64_t ntiles = a.nouter * a.ncolblocks;
   const int tid = threadIdx.y * W + threadIdx.x;
   uint32_t* rp = nullptr;
+  if constexpr (CHAIN) chain_next();
   if constexpr (strided_cache_rows(L)) {
     rp = strided_rowparts<L, W>(smem);
     strided_rowparts_init<L>(a, rp, tid, W * T);  // published by the first tile's barriers
   }
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
-    strided_tile<L, T, W, false, Rs...>(a, tile, smem, threadIdx.x, opaque_tid_y(), tid, rp);
+    strided_tile<L, T, W, false, CHAIN, Rs...>(a, tile, smem, threadIdx.x, opaque_tid_y(), tid, rp);
 }
 
 // the kernel's shared-memory limit raised to 227 KB, once per device
@@ -52,21 +57,24 @@ __global__ void __launch_bounds__(W * T, MB) k_strided_spec(const StridedArgs a)
 
 constexpr int64_t kMaxGrid = 1 << 20;
 
-template <int L, int T, int B, int MB, int... Rs>
+template <int L, int T, int B, int MB, bool CHAIN, int... Rs>
 cudaError_t run_contig(const ContigArgs& a, cudaStream_t s) {
-  TFFT_ALLOW_SMEM((k_contig_spec<L, T, B, MB, Rs...>));
+  if constexpr (!CHAIN && chainable(L))
+    if (a.chained) return run_contig<L, T, B, MB, true, Rs...>(a, s);
+  TFFT_ALLOW_SMEM((k_contig_spec<L, T, B, MB, CHAIN, Rs...>));
   if (attr != cudaSuccess) return attr;
   const size_t smem = (size_t)B * line_pitch<L, Rs...>() * sizeof(float2);
   int64_t grid = (a.nlines + B - 1) / B;
   if (grid > kMaxGrid) grid = kMaxGrid;
   if (grid < 1) return cudaSuccess;
-  k_contig_spec<L, T, B, MB, Rs...><<<(unsigned)grid, dim3(T, B), smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_chained(k_contig_spec<L, T, B, MB, CHAIN, Rs...>, dim3((unsigned)grid), dim3(T, B), smem, s, CHAIN ? a.chained : 0, a);
 }
 
-template <int L, int T, int W, int MB, int... Rs>
+template <int L, int T, int W, int MB, bool CHAIN, int... Rs>
 cudaError_t run_strided(const StridedArgs& a, cudaStream_t s) {
-  TFFT_ALLOW_SMEM((k_strided_spec<L, T, W, MB, Rs...>));
+  if constexpr (!CHAIN && chainable(L))
+    if (a.chained) return run_strided<L, T, W, MB, true, Rs...>(a, s);
+  TFFT_ALLOW_SMEM((k_strided_spec<L, T, W, MB, CHAIN, Rs...>));
   if (attr != cudaSuccess) return attr;
   if (a.W != W) return cudaErrorInvalidValue;
   constexpr size_t smem = strided_tile_smem<L, W>(strided_cache_rows(L));
@@ -75,14 +83,13 @@ cudaError_t run_strided(const StridedArgs& a, cudaStream_t s) {
   static PerDevice<int64_t> slots_cache;
   const int64_t slots = slots_cache.get(current_device(), [] {
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_strided_spec<L, T, W, MB, Rs...>, W * T, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_strided_spec<L, T, W, MB, CHAIN, Rs...>, W * T, smem);
     return (int64_t)device_sm_count() * (per_sm > 0 ? per_sm : 1);
   });
   int64_t grid = a.nouter * a.ncolblocks;
   if (grid > slots) grid = slots;
   if (grid < 1) return cudaSuccess;
-  k_strided_spec<L, T, W, MB, Rs...><<<(unsigned)grid, dim3(W, T), smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_chained(k_strided_spec<L, T, W, MB, CHAIN, Rs...>, dim3((unsigned)grid), dim3(W, T), smem, s, CHAIN ? a.chained : 0, a);
 }
 
 // The rows are compiled in kSpecParts translation units (tfft_spec_part.cu),

@@ -22,7 +22,7 @@ using namespace tiles;
 // z = backward FFT_L(Z), x[2n] = Re z[n], x[2n+1] = Im z[n]; the imaginary
 // parts of X[0] and X[L] are ignored (taken as zero).
 
-template <int L, int T, int B, int MB, int... Rs>
+template <int L, int T, int B, int MB, bool CHAIN, int... Rs>
 __global__ void __launch_bounds__(T * B, MB)
     k_r2c_spec(const RealArgs a) {
   constexpr int NST = sizeof...(Rs);
@@ -31,6 +31,10 @@ __global__ void __launch_bounds__(T * B, MB)
   extern __shared__ float2 smem[];
   const int ly = threadIdx.y;
   float2* sl = smem + ly * LP;
+  if constexpr (CHAIN) {
+    chain_next();
+    chain_wait();
+  }
   for (int64_t base = (int64_t)blockIdx.x * B; base < a.nlines; base += (int64_t)gridDim.x * B) {
     const int64_t line = base + ly;
     const bool act = line < a.nlines;
@@ -92,7 +96,7 @@ __global__ void __launch_bounds__(T * B, MB)
   }
 }
 
-template <int L, int T, int B, int MB, int... Rs>
+template <int L, int T, int B, int MB, bool CHAIN, int... Rs>
 __global__ void __launch_bounds__(T * B, MB)
     k_c2r_spec(const RealArgs a) {
   constexpr int NST = sizeof...(Rs);
@@ -101,6 +105,10 @@ __global__ void __launch_bounds__(T * B, MB)
   extern __shared__ float2 smem[];
   const int ly = threadIdx.y;
   float2* sl = smem + ly * LP;
+  if constexpr (CHAIN) {
+    chain_next();
+    chain_wait();
+  }
   for (int64_t base = (int64_t)blockIdx.x * B; base < a.nlines; base += (int64_t)gridDim.x * B) {
     const int64_t line = base + ly;
     const bool act = line < a.nlines;
@@ -193,23 +201,24 @@ __global__ void __launch_bounds__(T * B, MB)
 
 constexpr int64_t kMaxGrid = 1 << 20;
 
-template <int L, int T, int B, int MB, int... Rs>
+template <int L, int T, int B, int MB, bool CHAIN, int... Rs>
 cudaError_t run_real(const RealArgs& a, cudaStream_t s) {
+  if constexpr (!CHAIN && chainable(L))
+    if (a.chained) return run_real<L, T, B, MB, true, Rs...>(a, s);
   const int64_t grid0 = (a.nlines + B - 1) / B;
   const int64_t grid = grid0 > kMaxGrid ? kMaxGrid : grid0;
   if (grid < 1) return cudaSuccess;
   if (a.dir < 0) {
-    TFFT_ALLOW_SMEM((k_r2c_spec<L, T, B, MB, Rs...>));
+    TFFT_ALLOW_SMEM((k_r2c_spec<L, T, B, MB, CHAIN, Rs...>));
     if (attr != cudaSuccess) return attr;
     const size_t smem = (size_t)B * line_pitch<L, Rs...>() * sizeof(float2);
-    k_r2c_spec<L, T, B, MB, Rs...><<<(unsigned)grid, dim3(T, B), smem, s>>>(a);
+    return launch_chained(k_r2c_spec<L, T, B, MB, CHAIN, Rs...>, dim3((unsigned)grid), dim3(T, B), smem, s, CHAIN ? a.chained : 0, a);
   } else {
-    TFFT_ALLOW_SMEM((k_c2r_spec<L, T, B, MB, Rs...>));
+    TFFT_ALLOW_SMEM((k_c2r_spec<L, T, B, MB, CHAIN, Rs...>));
     if (attr != cudaSuccess) return attr;
     const size_t smem = (size_t)B * (line_pitch<L, Rs...>() + 1) * sizeof(float2);
-    k_c2r_spec<L, T, B, MB, Rs...><<<(unsigned)grid, dim3(T, B), smem, s>>>(a);
+    return launch_chained(k_c2r_spec<L, T, B, MB, CHAIN, Rs...>, dim3((unsigned)grid), dim3(T, B), smem, s, CHAIN ? a.chained : 0, a);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace
@@ -230,7 +239,7 @@ template <class Args>
 cudaError_t launch_real_row(const Args& a, cudaStream_t s) {
 #define X(LL, T, B, MB, ...)                                              \
   if constexpr (real_length(LL) && std::is_same<Args, RealArgs>::value) \
-    if (a.ap.L == LL) return run_real<LL, T, B, MB, __VA_ARGS__>(a, s);
+    if (a.ap.L == LL) return run_real<LL, T, B, MB, false, __VA_ARGS__>(a, s);
   TFFT_CONTIG_LINES(X)
 #undef X
   return cudaErrorInvalidValue;

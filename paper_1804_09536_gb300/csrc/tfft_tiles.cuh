@@ -84,52 +84,58 @@ __device__ __forceinline__ void spec_stage(float2 (&v)[EM], int jt, const float2
   }
 }
 
-// Twiddles of every stage after the first for one thread, held in registers.
-// They depend only on the thread's position in the line, so a persistent
-// kernel loads them once instead of once per tile.  Stage s (span Ns, radix
-// R) multiplies item r of butterfly q by w_L^{r (j % Ns) L / (Ns R)} with
-// j = jt + q T; the values are stored from offset(s) on, (R - 1) per q.
-template <int L, int E, int... Rs>
+// Twiddles of every stage after the first for one thread.  They depend only
+// on the thread's position in the line, so a persistent kernel loads them
+// into registers once instead of once per tile where they fit beside its
+// values: plans without guards and with at most 32 of them.  Others read
+// them per tile.  Stage s (span Ns, radix R) multiplies item r of butterfly q
+// by w_L^{r (j % Ns) L / (Ns R)} with j = jt + q T; the held values are
+// stored from offset(s) on, (R - 1) per q.
+template <int L, int T, int... Rs>
 struct StageTwiddles {
-  static_assert(((E % Rs == 0) && ...), "every radix divides E (uniform plans)");
   static constexpr int NST = sizeof...(Rs);
   __host__ __device__ static constexpr int offset(int s) {
     constexpr int r[] = {Rs...};
     int c = 0;
-    for (int i = 1; i < s; ++i) c += (E / r[i]) * (r[i] - 1);
+    for (int i = 1; i < s; ++i) c += (L / T / r[i]) * (r[i] - 1);
     return c;
   }
-  static constexpr int COUNT = offset(NST);
+  static constexpr bool HELD = (nbf_exact<L, T, Rs>() && ...) && offset(NST) <= 32;
+  static constexpr int COUNT = HELD ? offset(NST) : 0;
   float2 w[COUNT > 0 ? COUNT : 1];
 
   __device__ __forceinline__ void load(int jt, const float2* __restrict__ tw) {
-    constexpr int T = L / E;
-    static_for<1, NST>([&](auto S) {
-      constexpr int s = decltype(S)::value;
-      constexpr int R = radix_at<s, Rs...>();
-      constexpr int Ns = span_at<s, Rs...>();
-      constexpr int off = offset(s);
+    if constexpr (HELD)
+      static_for<1, NST>([&](auto S) {
+        constexpr int s = decltype(S)::value;
+        constexpr int R = radix_at<s, Rs...>();
+        constexpr int Ns = span_at<s, Rs...>();
+        constexpr int off = offset(s);
 #pragma unroll
-      for (int q = 0; q < E / R; ++q) {
-        const int step = ((jt + q * T) % Ns) * (L / (Ns * R));
+        for (int q = 0; q < L / T / R; ++q) {
+          const int step = ((jt + q * T) % Ns) * (L / (Ns * R));
 #pragma unroll
-        for (int r = 1; r < R; ++r) w[off + q * (R - 1) + r - 1] = __ldg(&tw[r * step]);
-      }
-    });
+          for (int r = 1; r < R; ++r) w[off + q * (R - 1) + r - 1] = __ldg(&tw[r * step]);
+        }
+      });
   }
 
-  // Stage s on a thread's items with the held twiddles.
-  template <int s>
-  __device__ __forceinline__ void stage(float2 (&v)[E]) const {
+  // Stage s on a thread's items.
+  template <int s, int EM>
+  __device__ __forceinline__ void stage(float2 (&v)[EM], int jt, const float2* __restrict__ tw) const {
     constexpr int R = radix_at<s, Rs...>();
-    constexpr int off = offset(s);
+    if constexpr (!HELD) {
+      spec_stage<L, T, R, span_at<s, Rs...>()>(v, jt, tw);
+    } else {
+      constexpr int off = offset(s);
 #pragma unroll
-    for (int q = 0; q < E / R; ++q) {
-      if constexpr (s > 0) {
+      for (int q = 0; q < L / T / R; ++q) {
+        if constexpr (s > 0) {
 #pragma unroll
-        for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], w[off + q * (R - 1) + r - 1]);
+          for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], w[off + q * (R - 1) + r - 1]);
+        }
+        Dft<R>::run(&v[q * R]);
       }
-      Dft<R>::run(&v[q * R]);
     }
   }
 };
@@ -325,7 +331,7 @@ __device__ __forceinline__ int row_offset(const DevLayout& lay, int axis, const 
 // column cx; tid = thread index in the CTA (W x T threads).  `rp` is the
 // per-CTA part/index table of strided_rowparts_init, or null (then each row
 // locates its part itself).
-template <int L, int T, int W, bool CG, int... Rs>
+template <int L, int T, int W, bool CG, bool CHAIN, int... Rs>
 __device__ __forceinline__ void strided_tile(const StridedArgs& a, int64_t tile, float2* smem, int cx, int jt,
                                              int tid, const uint32_t* rp = nullptr) {
   constexpr int NST = sizeof...(Rs);
@@ -365,6 +371,10 @@ __device__ __forceinline__ void strided_tile(const StridedArgs& a, int64_t tile,
   __syncthreads();
   const int2 blk = ts->blk;
   const bool act = cx < blk.y;
+  // the tables of a chained pass's first tile are built while the previous
+  // kernel drains
+  if constexpr (CHAIN)
+    if (tile == blockIdx.x) chain_wait();
   float2 v[emax<L, T, Rs...>()];
   static_for<0, NST>([&](auto S) {
     constexpr int s = decltype(S)::value;

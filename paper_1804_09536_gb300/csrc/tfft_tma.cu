@@ -72,6 +72,10 @@ __host__ __device__ constexpr size_t strided_tma_smem(int L, int W) {
 struct BlockTiles {
   CUtensorMap tin, tout;
   TmaGeo gin, gout;
+  __device__ __forceinline__ void prefetch() const {
+    tma_prefetch(&tin);
+    tma_prefetch(&tout);
+  }
   __host__ __device__ __forceinline__ int64_t ntiles(const StridedArgs& a) const { return a.nouter * a.ncolblocks; }
   template <int W>
   __device__ __forceinline__ void load(const StridedArgs& a, int64_t tile, float2* dst, uint64_t* bar) const {
@@ -107,6 +111,12 @@ struct BlockTiles {
 struct RankGroupTiles {
   CUtensorMap tin[kMaxRankGroups], tout[kMaxRankGroups];
   RankGroupGeo geo;
+  __device__ __forceinline__ void prefetch() const {
+    for (int g = 0; g < geo.ngroups; ++g) {
+      tma_prefetch(&tin[g]);
+      tma_prefetch(&tout[g]);
+    }
+  }
   __host__ __device__ __forceinline__ int64_t ntiles(const StridedArgs&) const { return geo.first[geo.ngroups]; }
   __device__ __forceinline__ int place(int64_t tile, int (&c)[5]) const {
     int g = 0;
@@ -135,10 +145,10 @@ struct RankGroupTiles {
   }
 };
 
-template <int L, int E, int W, class Geo, int... Rs>
-__global__ void __launch_bounds__(W * (L / E), strided_tma_ctas(strided_tma_smem(L, W)))
+template <int L, int T, int W, bool CHAIN, class Geo, int... Rs>
+__global__ void __launch_bounds__(W * T, strided_tma_ctas(strided_tma_smem(L, W)))
     k_strided_tma(const StridedArgs a, const __grid_constant__ Geo geo) {
-  constexpr int T = L / E, NST = sizeof...(Rs);
+  constexpr int NST = sizeof...(Rs);
   constexpr int WP = (W % 16 == 0) ? W : W + 1;  // exchange pitch (bank-conflict padding)
   constexpr int BUF = L * (W + 1);
   extern __shared__ __align__(128) float2 smem[];
@@ -157,8 +167,10 @@ __global__ void __launch_bounds__(W * (L / E), strided_tma_ctas(strided_tma_smem
     for (int b = 0; b < NB; ++b) mbar_init(&bars[b], 1);
     fence_mbar_init();
     fence_proxy_async();
+    if constexpr (CHAIN) geo.prefetch();
   }
   __syncthreads();
+  if constexpr (CHAIN) chain_next();
 
   auto issue_load = [&](int64_t tile, float2* dst, uint64_t* bar) {
     mbar_expect_tx(bar, tile_bytes);
@@ -166,9 +178,13 @@ __global__ void __launch_bounds__(W * (L / E), strided_tma_ctas(strided_tma_smem
   };
 
   int64_t tile = blockIdx.x;
+  StageTwiddles<L, T, Rs...> twr;
+  if constexpr (CHAIN) {
+    twr.load(threadIdx.y, a.tw);
+    chain_wait();
+  }
   if (tid == 0 && tile < ntiles) issue_load(tile, smem, &bars[0]);
-  StageTwiddles<L, E, Rs...> twr;
-  twr.load(threadIdx.y, a.tw);
+  if constexpr (!CHAIN) twr.load(threadIdx.y, a.tw);
   int it = 0, b = 0;  // b = it % NB
   for (; tile < ntiles; tile += gridDim.x, ++it, b = (b == NB - 1) ? 0 : b + 1) {
     float2* cur = smem + b * BUF;
@@ -194,47 +210,51 @@ __global__ void __launch_bounds__(W * (L / E), strided_tma_ctas(strided_tma_smem
       break;
     }
     const int jt = opaque_tid_y();
-    float2 v[E];
+    float2 v[emax<L, T, Rs...>()];
     static_for<0, NST>([&](auto S) {
       constexpr int s = decltype(S)::value;
       constexpr int R = radix_at<s, Rs...>();
       constexpr int Ns = span_at<s, Rs...>();
       if constexpr (s == 0) {
 #pragma unroll
-        for (int q = 0; q < E / R; ++q)
+        for (int q = 0; q < nbf<L, T, R>(); ++q)
+          if (bf_exists<L, T, R>(jt, q))
 #pragma unroll
-          for (int r = 0; r < R; ++r) {
-            float2 x = cur[(jt + q * T + r * (L / R)) * W + cx];
-            if (inv) x.y = -x.y;
-            v[q * R + r] = x;
-          }
+            for (int r = 0; r < R; ++r) {
+              float2 x = cur[(jt + q * T + r * (L / R)) * W + cx];
+              if (inv) x.y = -x.y;
+              v[q * R + r] = x;
+            }
       } else {
         constexpr int Rp = radix_at<s - 1, Rs...>();
         constexpr int Nsp = Ns / Rp;
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < E / Rp; ++q)
+        for (int q = 0; q < nbf<L, T, Rp>(); ++q)
+          if (bf_exists<L, T, Rp>(jt, q))
 #pragma unroll
-          for (int r = 0; r < Rp; ++r)
-            cur[stockham_out_index(jt + q * T, Nsp, Rp, r) * WP + cx] = v[q * Rp + r];
+            for (int r = 0; r < Rp; ++r)
+              cur[stockham_out_index(jt + q * T, Nsp, Rp, r) * WP + cx] = v[q * Rp + r];
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < E / R; ++q)
+        for (int q = 0; q < nbf<L, T, R>(); ++q)
+          if (bf_exists<L, T, R>(jt, q))
 #pragma unroll
-          for (int r = 0; r < R; ++r) v[q * R + r] = cur[(jt + q * T + r * (L / R)) * WP + cx];
+            for (int r = 0; r < R; ++r) v[q * R + r] = cur[(jt + q * T + r * (L / R)) * WP + cx];
       }
-      twr.template stage<s>(v);
+      twr.template stage<s>(v, jt, a.tw);
     });
     constexpr int RL = radix_at<NST - 1, Rs...>();
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < E / RL; ++q)
+    for (int q = 0; q < nbf<L, T, RL>(); ++q)
+      if (bf_exists<L, T, RL>(jt, q))
 #pragma unroll
-      for (int r = 0; r < RL; ++r) {
-        float2 x = cscale(v[q * RL + r], a.scale);
-        if (inv) x.y = -x.y;
-        cur[(jt + q * T + r * (L / RL)) * W + cx] = x;
-      }
+        for (int r = 0; r < RL; ++r) {
+          float2 x = cscale(v[q * RL + r], a.scale);
+          if (inv) x.y = -x.y;
+          cur[(jt + q * T + r * (L / RL)) * W + cx] = x;
+        }
     fence_proxy_async();
     __syncthreads();
     if (tid == 0) {
@@ -242,7 +262,9 @@ __global__ void __launch_bounds__(W * (L / E), strided_tma_ctas(strided_tma_smem
       bulk_commit();
     }
   }
-  if (tid == 0) bulk_wait_all();
+  // the stores have read their tile buffers; the writes themselves complete
+  // before the grid does
+  if (tid == 0) bulk_wait_read<0>();
 }
 
 // the kernel's shared-memory limit raised to 227 KB, once per device
@@ -259,52 +281,58 @@ int64_t persistent_grid(K kernel, int threads, size_t smem, int64_t ntiles) {
   return ntiles < g ? ntiles : g;
 }
 
-template <int L, int E, int W, class Geo, int... Rs>
+template <int L, int T, int W, bool CHAIN, class Geo, int... Rs>
 cudaError_t run_strided_tma(const StridedArgs& a, const Geo& geo, cudaStream_t s) {
-  auto kern = k_strided_tma<L, E, W, Geo, Rs...>;
+  if constexpr (!CHAIN && chainable(L))
+    if (a.chained) return run_strided_tma<L, T, W, true, Geo, Rs...>(a, geo, s);
+  if (a.W != W) return cudaErrorInvalidValue;
+  auto kern = k_strided_tma<L, T, W, CHAIN, Geo, Rs...>;
   TFFT_ALLOW_SMEM(kern);
   if (attr != cudaSuccess) return attr;
-  if (a.W != W) return cudaErrorInvalidValue;
   const size_t smem = strided_tma_smem(L, W);
-  const int threads = W * (L / E);
+  const int threads = W * T;
   static PerDevice<int64_t> slots_cache;
   const int64_t slots =
       slots_cache.get(current_device(), [&] { return persistent_grid(kern, threads, smem, int64_t(1) << 40); });
   const int64_t ntiles = geo.ntiles(a);
   const int64_t grid = ntiles < slots ? ntiles : slots;
   if (grid < 1) return cudaSuccess;
-  kern<<<(unsigned)grid, dim3(W, L / E), smem, s>>>(a, geo);
-  return cudaGetLastError();
+  return launch_chained(kern, dim3((unsigned)grid), dim3(W, T), smem, s, CHAIN ? a.chained : 0, a, geo);
 }
 
-// Strided TMA variants: length, elements per thread, tile width, radices.
-// The first row of a length is its default; tma_strided_variant() can pick
-// another (autotuning).  256: 16-column tiles at two CTAs per SM beat 32
-// columns at one (256^3 on 4 x 8 / 2 x 2 / 2 x 4: 0.048 vs 0.052 ms per pass;
-// the 48-transform batch 1.96 vs 2.01 ms); 8 elements per thread (radices
-// 8, 8, 4) took 0.057 ms.  512: 8-column tiles at two CTAs per SM took 0.361
+// Strided TMA variants: length, threads per column, tile width, radices (the
+// plain pass's, so that the two agree bit for bit; 512 excepted).  A plan
+// takes the first row of its length whose width divides every rank's columns;
+// the environment can ask for another (tuning).
+// 96 (8.12), 160 (16.10) and 384 (16.24) cross shared memory once where
+// 4.4.3.2, 5.4.4.2 and 8.8.3.2 crossed it three times: 96 x 96 x 512 20.5 ->
+// 16.4 us, 160 x 160 x 512 47 -> 41 us, 384^3 192 -> 153 us per pass.
+// 256: 16-column tiles beat 32 columns (256^3 on 4 x 8 / 2 x 2 / 2 x 4: 0.048
+// vs 0.052 ms per pass; the 48-transform batch 1.96 vs 2.01 ms); radices
+// 8, 8, 4 took 0.057 ms.  512: 8-column tiles at two CTAs per SM took 0.361
 // vs 0.336 ms per 512^3 pass (64-byte rows).
 #define TFFT_TMA_STRIDED(X)     \
   X(64, 8, 32, 8, 8)            \
-  X(96, 12, 32, 4, 4, 3, 2)     \
-  X(128, 16, 32, 16, 8)         \
-  X(160, 20, 16, 5, 4, 4, 2)    \
-  X(384, 24, 16, 8, 8, 3, 2)    \
+  X(96, 4, 32, 8, 12)           \
+  X(96, 12, 16, 8, 12)          \
+  X(128, 8, 32, 16, 8)          \
+  X(160, 16, 16, 16, 10)        \
+  X(384, 24, 16, 16, 24)        \
   X(1024, 32, 8, 32, 32)        \
   X(256, 16, 16, 16, 16)        \
   X(256, 16, 32, 16, 16)        \
-  X(512, 32, 16, 32, 16)        \
-  X(512, 16, 16, 8, 8, 8)
+  X(512, 16, 16, 32, 16)        \
+  X(512, 32, 16, 8, 8, 8)
 
 }  // namespace
 
-bool tma_strided_variant(int L, int want_W, int want_E, int& E, int& W) {
+bool tma_strided_variant(int L, int want_W, int want_T, int& T, int& W) {
   bool found = false;
-#define X(LL, EE, WW, ...)                                             \
+#define X(LL, TT, WW, ...)                                             \
   if (LL == L) {                                                        \
-    const bool match = WW == want_W && (want_E == 0 || EE == want_E);  \
+    const bool match = WW == want_W && (want_T == 0 || TT == want_T);  \
     if (!found || match) {                                              \
-      E = EE;                                                           \
+      T = TT;                                                           \
       W = WW;                                                           \
       found = true;                                                     \
       if (match) return true;                                           \
@@ -315,22 +343,34 @@ bool tma_strided_variant(int L, int want_W, int want_E, int& E, int& W) {
   return found;
 }
 
-cudaError_t launch_strided_tma(const StridedArgs& a, int E, const TmaGeo& gi, const TmaGeo& go,
+bool tma_strided_row(int L, int k, int& T, int& W) {
+#define X(LL, TT, WW, ...)    \
+  if (LL == L && k-- == 0) {  \
+    T = TT;                   \
+    W = WW;                   \
+    return true;              \
+  }
+  TFFT_TMA_STRIDED(X)
+#undef X
+  return false;
+}
+
+cudaError_t launch_strided_tma(const StridedArgs& a, int T, const TmaGeo& gi, const TmaGeo& go,
                                const void* tmap_in, const void* tmap_out, cudaStream_t s) {
   BlockTiles geo;
   geo.tin = *static_cast<const CUtensorMap*>(tmap_in);
   geo.tout = *static_cast<const CUtensorMap*>(tmap_out);
   geo.gin = gi;
   geo.gout = go;
-#define X(LL, EE, WW, ...)                   \
-  if (a.ap.L == LL && E == EE && a.W == WW) \
-    return run_strided_tma<LL, EE, WW, BlockTiles, __VA_ARGS__>(a, geo, s);
+#define X(LL, TT, WW, ...)                   \
+  if (a.ap.L == LL && T == TT && a.W == WW) \
+    return run_strided_tma<LL, TT, WW, false, BlockTiles, __VA_ARGS__>(a, geo, s);
   TFFT_TMA_STRIDED(X)
 #undef X
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_strided_tma_groups(const StridedArgs& a, int E, const RankGroupGeo& g, const void* const* tmaps_in,
+cudaError_t launch_strided_tma_groups(const StridedArgs& a, int T, const RankGroupGeo& g, const void* const* tmaps_in,
                                       const void* const* tmaps_out, cudaStream_t s) {
   if (g.ngroups < 1 || g.ngroups > kMaxRankGroups || g.width != a.W) return cudaErrorInvalidValue;
   RankGroupTiles geo;
@@ -339,9 +379,9 @@ cudaError_t launch_strided_tma_groups(const StridedArgs& a, int E, const RankGro
     geo.tout[k] = *static_cast<const CUtensorMap*>(tmaps_out[k]);
   }
   geo.geo = g;
-#define X(LL, EE, WW, ...)                   \
-  if (a.ap.L == LL && E == EE && a.W == WW) \
-    return run_strided_tma<LL, EE, WW, RankGroupTiles, __VA_ARGS__>(a, geo, s);
+#define X(LL, TT, WW, ...)                   \
+  if (a.ap.L == LL && T == TT && a.W == WW) \
+    return run_strided_tma<LL, TT, WW, false, RankGroupTiles, __VA_ARGS__>(a, geo, s);
   TFFT_TMA_STRIDED(X)
 #undef X
   return cudaErrorInvalidValue;

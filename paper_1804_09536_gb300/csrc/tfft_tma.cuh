@@ -84,6 +84,11 @@ __device__ __forceinline__ void tma_store_5d(const CUtensorMap* map, const void*
       : "memory");
 }
 
+// Fetches a tensor map ahead of its first copy.
+__device__ __forceinline__ void tma_prefetch(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
+
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 
 template <int N>

@@ -106,11 +106,11 @@ bool encode_stage_map(tfft_plan p, const TmaGeo& G, int axis, int W, const void*
   return r == CUDA_SUCCESS;
 }
 
-// Tile width (and optionally elements per thread) requested for the strided
+// Tile width (and optionally threads per column) requested for the strided
 // TMA pass of length L by the environment, TFFT_TMA_W="512:8:16,256:32"
 // (TFFT_TC_W for the tensor-core passes; used when tuning); 0 when not given.
-int tuned_width(int L, int* E, const char* var) {
-  if (E) *E = 0;
+int tuned_width(int L, int* T, const char* var) {
+  if (T) *T = 0;
   const char* env = std::getenv(var);
   if (!env) return 0;
   std::string v(env);
@@ -121,7 +121,7 @@ int tuned_width(int L, int* E, const char* var) {
     size_t colon = item.find(':');
     if (colon != std::string::npos && std::atoi(item.substr(0, colon).c_str()) == L) {
       size_t colon2 = item.find(':', colon + 1);
-      if (E && colon2 != std::string::npos) *E = std::atoi(item.substr(colon2 + 1).c_str());
+      if (T && colon2 != std::string::npos) *T = std::atoi(item.substr(colon2 + 1).c_str());
       return std::atoi(item.substr(colon + 1).c_str());
     }
     if (comma == std::string::npos) break;
@@ -363,9 +363,9 @@ bool plan_padding(tfft_plan p) {
   const int L = (int)p->cshape[ax];
   auto it = p->aplan_s.find(L);
   if (it == p->aplan_s.end() || !it->second.spec) return false;
-  int wantE = 0, Et = 0, Wt = 0;
-  const int wantW = tuned_width(L, &wantE);
-  if (!tma_strided_variant(L, wantW, wantE, Et, Wt)) return false;
+  int wantT = 0, Tt = 0, Wt = 0;
+  const int wantW = tuned_width(L, &wantT);
+  if (!tma_strided_variant(L, wantW, wantT, Tt, Wt)) return false;
   TmaGeo a{}, b{};
   if (tma_geo(p, 0, ax, Wt, a) && tma_geo(p, p->g, ax, Wt, b)) return false;  // no padding needed
   const LayoutH& S = p->st[p->g];
@@ -410,7 +410,7 @@ bool plan_padding(tfft_plan p) {
   p->pad_lead = lead;
   p->win_c0 = c0;
   p->win_nc = nc;
-  p->win_E = Et;
+  p->win_T = Tt;
   p->win_W = Wt;
   return true;
 }
