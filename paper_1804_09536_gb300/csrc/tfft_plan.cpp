@@ -209,13 +209,15 @@ bool is_smooth_235(int64_t n) {
   return n == 1;
 }
 
-// Bluestein plan for a length N without a 2/3/5 factorisation: convolution
-// length M = the power of two >= 2N - 1 (at most MAXLEN), and the tables,
+// Bluestein plan for a length N without a compiled factorisation: convolution
+// length M = the smallest compiled one >= 2N - 1, or the power of two where
+// the compiled passes do not apply (at most MAXLEN), and the tables,
 // evaluated in double and rounded once: chirp[n] = exp(-i pi (n^2 mod 2N) / N)
 // and bhat = FFT_M(b) / M for the wrapped filter b[m] = b[M - m] = conj(chirp[m]).
 bool make_bluestein(tfft_plan p, int N) {
   int M = 1;
   while (M < 2 * N - 1) M <<= 1;
+  if (M > 16 && p->nelems < (int64_t(1) << 31) && blue_spec_length(N) > 0) M = blue_spec_length(N);
   AxisPlan apm{};
   if (M > MAXLEN || !make_axis_plan(M, false, apm)) return false;
   const double pi = 3.14159265358979323846;

@@ -30,15 +30,6 @@ bool row_plan(const SpecRow& r, AxisPlan& ap, int& width) {
   return true;
 }
 
-// calls f(integral_constant<P>) for P == p
-template <int P = 0, class F>
-cudaError_t with_part(int p, F&& f) {
-  if constexpr (P < spec::kSpecParts)
-    return p == P ? f(std::integral_constant<int, P>{}) : with_part<P + 1>(p, f);
-  else
-    return cudaErrorInvalidValue;
-}
-
 }  // namespace
 
 bool spec_plan(int L, bool strided, int64_t nelems, AxisPlan& ap, int& width) {
@@ -62,12 +53,12 @@ bool real_plan(int L, int64_t nelems, AxisPlan& ap, int& width) {
 }
 
 cudaError_t launch_contig_spec(const ContigArgs& a, cudaStream_t s) {
-  return with_part(a.ap.L % spec::kSpecParts,
+  return spec::with_part(a.ap.L % spec::kSpecParts,
                    [&](auto p) { return spec::contig_part<decltype(p)::value>(a, s); });
 }
 
 cudaError_t launch_strided_spec(const StridedArgs& a, cudaStream_t s) {
-  return with_part(a.ap.L % spec::kSpecParts,
+  return spec::with_part(a.ap.L % spec::kSpecParts,
                    [&](auto p) { return spec::strided_part<decltype(p)::value>(a, s); });
 }
 

@@ -1,5 +1,7 @@
-// One part of the specialised passes: the rows L of tfft_spec_table.h with
-// L mod kSpecParts == TFFT_SPEC_PART (set by the build).
+// One part of the specialised passes: the rows L of tfft_spec_table.h, and the
+// convolution lengths M of tfft_blue.cuh, with L (M) mod kSpecParts ==
+// TFFT_SPEC_PART (set by the build).
+#include "tfft_blue.cuh"
 #include "tfft_spec_pass.cuh"
 
 namespace tfft {
@@ -29,4 +31,31 @@ template cudaError_t contig_part<TFFT_SPEC_PART>(const ContigArgs& a, cudaStream
 template cudaError_t strided_part<TFFT_SPEC_PART>(const StridedArgs& a, cudaStream_t s);
 
 }  // namespace spec
+
+namespace blue {
+
+template <int P>
+cudaError_t blue_contig_part(const ContigArgs& a, const BlueArgs& b, cudaStream_t s) {
+#define X(MM, T, B, MB, ...)                  \
+  if constexpr (MM % spec::kSpecParts == P)   \
+    if (b.M == MM) return run_blue_contig<MM, T, B, MB, __VA_ARGS__>(a, b, s);
+  TFFT_BLUE_CONTIG(X)
+#undef X
+  return cudaErrorInvalidValue;
+}
+
+template <int P>
+cudaError_t blue_strided_part(const StridedArgs& a, const BlueArgs& b, cudaStream_t s) {
+#define X(MM, T, W, MB, ...)                  \
+  if constexpr (MM % spec::kSpecParts == P)   \
+    if (b.M == MM) return run_blue_strided<MM, T, W, MB, __VA_ARGS__>(a, b, s);
+  TFFT_BLUE_STRIDED(X)
+#undef X
+  return cudaErrorInvalidValue;
+}
+
+template cudaError_t blue_contig_part<TFFT_SPEC_PART>(const ContigArgs& a, const BlueArgs& b, cudaStream_t s);
+template cudaError_t blue_strided_part<TFFT_SPEC_PART>(const StridedArgs& a, const BlueArgs& b, cudaStream_t s);
+
+}  // namespace blue
 }  // namespace tfft

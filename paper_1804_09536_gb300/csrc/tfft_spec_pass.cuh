@@ -92,10 +92,21 @@ cudaError_t run_strided(const StridedArgs& a, cudaStream_t s) {
   return launch_chained(k_strided_spec<L, T, W, MB, CHAIN, Rs...>, dim3((unsigned)grid), dim3(W, T), smem, s, CHAIN ? a.chained : 0, a);
 }
 
+#undef TFFT_ALLOW_SMEM
+
 // The rows are compiled in kSpecParts translation units (tfft_spec_part.cu),
 // row L in part L mod kSpecParts (a prime above 7 spreads the 2/3/5/7 lengths
 // evenly).
 constexpr int kSpecParts = 11;
+
+// calls f(integral_constant<P>) for P == p
+template <int P = 0, class F>
+cudaError_t with_part(int p, F&& f) {
+  if constexpr (P < kSpecParts)
+    return p == P ? f(std::integral_constant<int, P>{}) : with_part<P + 1>(p, f);
+  else
+    return cudaErrorInvalidValue;
+}
 
 template <int P>
 cudaError_t contig_part(const ContigArgs& a, cudaStream_t s);

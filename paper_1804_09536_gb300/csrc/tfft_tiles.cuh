@@ -154,13 +154,6 @@ __device__ __forceinline__ int opaque_tid_y() {
   return v;
 }
 
-// CTAs per SM the register budget is sized for: `target` resident threads
-// (half that for the 20-element plans, whose butterflies need more registers).
-__host__ __device__ constexpr int min_blocks(int E, int threads, int target) {
-  const int t = (E >= 20 ? target / 2 : target) / threads;
-  return t > 1 ? t : (E >= 20 && threads <= 256 ? 2 : 1);
-}
-
 // Synchronises the threads of one line: a warp when the line's threads lie
 // inside one (T divides 32), the whole CTA otherwise.
 template <int T>
