@@ -141,6 +141,7 @@ int batch_upload(tfft_batch b, cudaStream_t st) {
       a.nlines = s.nlines;
       a.ap = ap;
       a.tw = reinterpret_cast<const float2*>(p->d_state + p->tw_off[s.L]);
+      a.tws = nullptr;
       a.lines_per_cta = bw;
       a.sign = s.sign;
       a.scale = scale;

@@ -24,6 +24,15 @@ bool blue_spec_plan(int M, int& lines_per_cta, int& tile_width) {
   return c && t;
 }
 
+void blue_spec_radices(int M, int& nst, int* radix) {
+  nst = 0;
+#define X(MM, T, B, MB, ...)                  \
+  if (M == MM)                                \
+    for (int r : {__VA_ARGS__}) radix[nst++] = r;
+  TFFT_BLUE_CONTIG(X)
+#undef X
+}
+
 int blue_spec_length(int N) {
   int best = 0;
 #define X(MM, ...) \

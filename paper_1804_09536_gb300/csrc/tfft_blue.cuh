@@ -113,9 +113,9 @@ __global__ void __launch_bounds__(T * B, MB) k_blue_contig_spec(const ContigArgs
         }
         v[q * R0 + r] = x;
       }
-    stages<M, T, 0, false>(Radices<Rs...>{}, v, sl, 0, jt, b.twm);
+    stages<M, T, 0, false>(Radices<Rs...>{}, v, sl, 0, jt, b.tws_f);
     apply_filter<M, T, RL>(v, jt, b.bhat);
-    stages<M, T, 0, false>(Rev{}, v, sl, 0, jt, b.twm);
+    stages<M, T, 0, false>(Rev{}, v, sl, 0, jt, b.tws_r);
 #pragma unroll
     for (int q = 0; q < nbf<M, T, R0>(); ++q)
 #pragma unroll

@@ -35,6 +35,7 @@ struct ContigArgs {
   int64_t nlines;
   AxisPlan ap;
   const float2* tw;  // ap.L roots exp(-2 pi i m / L)
+  const float2* tws; // stage table of ap's radices (specialised passes)
   int lines_per_cta;
   int sign;
   float scale;
@@ -51,6 +52,8 @@ struct BlueArgs {
   int N, M;
   AxisPlan apm;          // length-M FFT plan (shared-memory stages)
   const float2* twm;     // the M roots exp(-2 pi i m / M)
+  const float2* tws_f;   // stage tables of the contiguous pass's two FFTs
+  const float2* tws_r;
   const float2* chirp;   // N values exp(-i pi (n^2 mod 2N) / N)
   const float2* bhat;    // M values: the FFT of the wrapped chirp filter, times 1 / M
 };
@@ -109,6 +112,7 @@ struct RealArgs {
   int64_t nlines;
   AxisPlan ap;          // plan of the length-L complex FFT
   const float2* tw;     // L roots exp(-2 pi i m / L)
+  const float2* tws;    // stage table of ap's radices
   const float2* tw2;    // 2L roots exp(-2 pi i m / 2L)
   int64_t cpitch;       // complex elements from one line's start to the next (>= L + 1)
   int dir;
@@ -290,11 +294,18 @@ cudaError_t launch_strided_blue(const StridedArgs& a, const BlueArgs& b, cudaStr
 // Bluestein passes with a compile-time convolution length (tfft_blue.cu):
 // whether M has them, and their lines per CTA and strided tile width.
 bool blue_spec_plan(int M, int& lines_per_cta, int& tile_width);
+// Radices of the contiguous pass of convolution length M.
+void blue_spec_radices(int M, int& nst, int* radix);
 // The compiled convolution length for lines of length N (0: none).
 int blue_spec_length(int N);
 cudaError_t launch_contig_blue_spec(const ContigArgs& a, const BlueArgs& b, cudaStream_t s);
 cudaError_t launch_strided_blue_spec(const StridedArgs& a, const BlueArgs& b, cudaStream_t s);
 cudaError_t launch_twiddles(float2* tw, int L, cudaStream_t s);
+// Stage table of a length-L plan (L entries reserved): for every stage after
+// the first (span Ns, radix R) the twiddles exp(-2 pi i r k / (Ns R)), r = 1 ..
+// R - 1, k = 0 .. Ns - 1, k fastest -- the values of the root table in the
+// order the contiguous passes read them.
+cudaError_t launch_stage_twiddles(float2* tws, int L, int nst, const int* radix, cudaStream_t s);
 
 // Batched persistent executor (tfft_batch.cu).  One segment = the tiles of
 // one pass of one transform; items are numbered consecutively over the

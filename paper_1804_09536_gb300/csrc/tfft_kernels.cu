@@ -486,6 +486,28 @@ __global__ void k_twiddles(float2* tw, int L) {
   }
 }
 
+struct StageRadices {
+  int n, r[MAXSTAGES];
+};
+
+__global__ void k_stage_twiddles(float2* tws, int L, const StageRadices p) {
+  int i = blockIdx.x * blockDim.x + threadIdx.x;
+  float2* out = tws + i;
+  int Ns = p.r[0];
+  for (int s = 1; s < p.n; ++s) {
+    const int R = p.r[s], n = (R - 1) * Ns;
+    if (i < n) {
+      const int m = (i / Ns + 1) * (i % Ns) * (L / (Ns * R));
+      double sn, cs;
+      sincospi(2.0 * (double)m / (double)L, &sn, &cs);
+      *out = make_float2((float)cs, (float)(-sn));
+      return;
+    }
+    i -= n;
+    Ns *= R;
+  }
+}
+
 // the kernel's shared-memory limit raised to 227 KB, once per device
 #define TFFT_ALLOW_SMEM(kernel)                          \
   static PerDevice<cudaError_t> attr_cache;              \
@@ -633,6 +655,14 @@ int device_sm_count() {
     if (dev < 0 || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) v = 0;
     return v > 0 ? v : 1;
   });
+}
+
+cudaError_t launch_stage_twiddles(float2* tws, int L, int nst, const int* radix, cudaStream_t s) {
+  StageRadices p = {};
+  p.n = nst;
+  for (int i = 0; i < nst; ++i) p.r[i] = radix[i];
+  k_stage_twiddles<<<(L + 255) / 256, 256, 0, s>>>(tws, L, p);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_twiddles(float2* tw, int L, cudaStream_t s) {

@@ -262,11 +262,28 @@ bool make_bluestein(tfft_plan p, int N) {
     ap.blue_spec = aps.blue_spec = 1;
     ap.width = spec_lines;
     aps.width = spec_w;
+    int nst = 0, radix[MAXSTAGES];
+    blue_spec_radices(M, nst, radix);
+    std::vector<int> f(radix, radix + nst);
+    add_stage_table(p, f);
+    add_stage_table(p, std::vector<int>(f.rbegin(), f.rend()));
   }
   p->aplan[N] = ap;
   p->aplan_s[N] = aps;
   p->blue[N] = h;
   return true;
+}
+
+// The stage table of a radix sequence: L entries of the plan state.
+void add_stage_table(tfft_plan p, std::vector<int> radices) {
+  int64_t L = 1;
+  for (int r : radices) L *= r;
+  if (!p->tws_off.count(radices)) p->tws_off[radices] = image_add(p, nullptr, (size_t)L * sizeof(float2));
+}
+
+const float2* stage_table(tfft_plan p, const AxisPlan& ap) {
+  auto it = p->tws_off.find(std::vector<int>(ap.radix, ap.radix + ap.nst));
+  return it == p->tws_off.end() ? nullptr : reinterpret_cast<const float2*>(p->d_state + it->second);
 }
 
 BlueArgs blue_args(tfft_plan p, int N) {
@@ -276,6 +293,15 @@ BlueArgs blue_args(tfft_plan p, int N) {
   b.M = h.M;
   b.apm = h.apm;
   b.twm = reinterpret_cast<const float2*>(p->d_state + p->tw_off.at(h.M));
+  b.tws_f = b.tws_r = nullptr;
+  if (p->aplan.at(N).blue_spec) {
+    AxisPlan f{}, r{};
+    blue_spec_radices(h.M, f.nst, f.radix);
+    r.nst = f.nst;
+    for (int i = 0; i < f.nst; ++i) r.radix[i] = f.radix[f.nst - 1 - i];
+    b.tws_f = stage_table(p, f);
+    b.tws_r = stage_table(p, r);
+  }
   b.chirp = reinterpret_cast<const float2*>(p->d_state + h.chirp_off);
   b.bhat = reinterpret_cast<const float2*>(p->d_state + h.bhat_off);
   return b;
@@ -387,6 +413,7 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
       p->rplan = AxisPlan{};
       if (real_plan(Lh, p->nelems, p->rplan, width)) {
         p->rplan.width = width;
+        add_stage_table(p, std::vector<int>(p->rplan.radix, p->rplan.radix + p->rplan.nst));
         if (!p->tw_off.count(Lh)) p->tw_off[Lh] = image_add(p, nullptr, (size_t)Lh * sizeof(float2));
         if (!p->tw_off.count(2 * Lh)) p->tw_off[2 * Lh] = image_add(p, nullptr, (size_t)2 * Lh * sizeof(float2));
       } else {
@@ -409,6 +436,7 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
         p->aplan[L] = ap;
         p->aplan_s[L] = aps;
         if (!p->tw_off.count(L)) p->tw_off[L] = image_add(p, nullptr, (size_t)L * sizeof(float2));
+        add_stage_table(p, std::vector<int>(ap.radix, ap.radix + ap.nst));
         continue;
       }
       if (!is_smooth_235(L) && L <= MAXLEN / 2) {
@@ -421,7 +449,10 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
         continue;
       }
       int width = 0;
-      if (spec_plan(L, false, p->nelems, ap, width)) ap.width = width;
+      if (spec_plan(L, false, p->nelems, ap, width)) {
+        ap.width = width;
+        add_stage_table(p, std::vector<int>(ap.radix, ap.radix + ap.nst));
+      }
       if (spec_plan(L, true, p->nelems, aps, width)) aps.width = width;
       p->aplan[L] = ap;
       p->aplan_s[L] = aps;
@@ -539,6 +570,13 @@ int tfft_plan_bind(tfft_plan p, void* d_state, size_t bytes, void* stream) {
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync (plan state)");
     for (auto& kv : p->tw_off) {
       e = launch_twiddles(reinterpret_cast<float2*>(static_cast<char*>(d_state) + kv.second), kv.first, st);
+      if (e != cudaSuccess) return cuda_fail(e, "twiddle generation");
+    }
+    for (auto& kv : p->tws_off) {
+      int L = 1;
+      for (int r : kv.first) L *= r;
+      e = launch_stage_twiddles(reinterpret_cast<float2*>(static_cast<char*>(d_state) + kv.second), L,
+                                (int)kv.first.size(), kv.first.data(), st);
       if (e != cudaSuccess) return cuda_fail(e, "twiddle generation");
     }
     e = cudaStreamSynchronize(st);

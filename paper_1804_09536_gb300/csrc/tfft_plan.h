@@ -176,6 +176,7 @@ struct tfft_plan_s {
   std::map<int, AxisPlan> aplan;   // contiguous-line passes
   std::map<int, AxisPlan> aplan_s; // strided passes
   std::map<int, size_t> tw_off;
+  std::map<std::vector<int>, size_t> tws_off;  // stage tables by their radices
   struct BlueH {       // Bluestein lengths: convolution plan and the offsets of their tables
     int M = 0;
     AxisPlan apm{};
@@ -265,6 +266,8 @@ int strided_width(const AxisPlan& ap);
 bool is_smooth_235(int64_t n);
 bool make_bluestein(tfft_plan p, int N);
 BlueArgs blue_args(tfft_plan p, int N);
+void add_stage_table(tfft_plan p, std::vector<int> radices);
+const float2* stage_table(tfft_plan p, const AxisPlan& ap);
 int check_ptr(const void* ptr, const char* name);
 int check_bound(tfft_plan p);
 

@@ -22,6 +22,34 @@ using namespace tiles;
 // z = backward FFT_L(Z), x[2n] = Re z[n], x[2n+1] = Im z[n]; the imaginary
 // parts of X[0] and X[L] are ignored (taken as zero).
 
+// How the lines' Hermitian halves are spread over threads: the threads that
+// synchronise together (a warp with 32 / T lines, or a line's T > 32 threads)
+// take the pairs (k, L - k), k < L/2, of their lines in order, so that a warp
+// reads or writes 32 consecutive elements of one row each way.  With T = 8
+// threads a row, four rows per request in 64-byte pieces, the L1 was the
+// bound (85 % busy in the c2r pass of 256^3, 45 % of its shared wavefronts
+// bank conflicts).
+template <int L, int T>
+struct RealGroup {
+  static constexpr int G = T > 32 ? T : 32;  // threads of a group
+  static constexpr int LINES = G / T;
+  static constexpr int NPAIR = (LINES * (L / 2) + G - 1) / G;
+  static_assert(L % 2 == 0 && G % T == 0, "even lengths, whole lines");
+  int lane, first;  // thread in the group, the group's first line in the CTA
+  __device__ __forceinline__ RealGroup(int ly, int jt) {
+    const unsigned tid = (unsigned)(ly * T + jt);
+    lane = (int)(tid % G);
+    first = (int)(tid / G) * LINES;
+  }
+  // Pair n of this thread: line i of the group and k; false past the end.
+  __device__ __forceinline__ bool pair(int n, int& i, int& k) const {
+    const unsigned u = (unsigned)(lane + n * G);
+    i = (int)(u / (L / 2));
+    k = (int)(u % (L / 2));
+    return LINES * (L / 2) % G == 0 || u < (unsigned)(LINES * (L / 2));
+  }
+};
+
 template <int L, int T, int B, int MB, bool CHAIN, int... Rs>
 __global__ void __launch_bounds__(T * B, MB)
     k_r2c_spec(const RealArgs a) {
@@ -39,7 +67,6 @@ __global__ void __launch_bounds__(T * B, MB)
     const int64_t line = base + ly;
     const bool act = line < a.nlines;
     const float2* src = reinterpret_cast<const float2*>(a.rin) + line * L;
-    float2* dst = a.cout + line * a.cpitch;
     const int jt = opaque_tid_x();
     float2 v[emax<L, T, Rs...>()];
     static_for<0, NST>([&](auto S) {
@@ -68,7 +95,8 @@ __global__ void __launch_bounds__(T * B, MB)
 #pragma unroll
             for (int r = 0; r < R; ++r) v[q * R + r] = sl[padp<P>(jt + q * T + r * (L / R))];
       }
-      spec_stage<L, T, R, Ns>(v, jt, a.tw);
+      constexpr int OFF = stage_table_off<s, Rs...>();
+      spec_stage<L, T, R, Ns, OFF>(v, jt, OFF < 0 ? a.tw : a.tws);
     });
     constexpr int RL = radix_at<NST - 1, Rs...>();
     line_sync<T>();
@@ -82,16 +110,34 @@ __global__ void __launch_bounds__(T * B, MB)
     // w^(L-k) = -conj(w^k) and the roles of Z[k], Z[L-k] swap,
     // X[L-k] = conj(e - o) -- one pair of shared loads and one twiddle for two
     // outputs (k = 0 gives X[0] and X[L]; k = L/2 is its own partner)
-    for (int k = jt; k <= L / 2; k += T) {
-      const float2 zk = sl[padp<P>(k)];
-      const float2 zm = sl[padp<P>(k == 0 ? 0 : L - k)];
+    const RealGroup<L, T> g(ly, jt);
+    const int64_t gline = base + g.first;
+    auto pair = [&](int i, int k, float2& lo, float2& hi) {
+      const float2* z = smem + (g.first + i) * LP;
+      const float2 zk = z[padp<P>(k)];
+      const float2 zm = z[padp<P>(k == 0 ? 0 : L - k)];
       const float2 e = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));   // (Z[k] + conj Z[L-k]) / 2
       const float2 d = make_float2(0.5f * (zk.x - zm.x), 0.5f * (zk.y + zm.y));   // (Z[k] - conj Z[L-k]) / 2
       const float2 o = cmul(__ldg(&a.tw2[k]), mul_mi(d));                          // -i w^k d
-      if (act) {
-        dst[k] = cscale(cadd(e, o), a.scale);
-        if (2 * k != L) dst[L - k] = cscale(make_float2(e.x - o.x, o.y - e.y), a.scale);
+      lo = cscale(cadd(e, o), a.scale);
+      hi = cscale(make_float2(e.x - o.x, o.y - e.y), a.scale);
+    };
+#pragma unroll
+    for (int n = 0; n < g.NPAIR; ++n) {
+      int i, k;
+      if (!g.pair(n, i, k)) continue;
+      float2 lo, hi;
+      pair(i, k, lo, hi);
+      if (gline + i < a.nlines) {
+        float2* row = a.cout + (gline + i) * a.cpitch;
+        row[k] = lo;
+        row[L - k] = hi;
       }
+    }
+    if (g.lane < g.LINES && gline + g.lane < a.nlines) {
+      float2 lo, hi;
+      pair(g.lane, L / 2, lo, hi);
+      a.cout[(gline + g.lane) * a.cpitch + L / 2] = lo;
     }
   }
 }
@@ -112,45 +158,51 @@ __global__ void __launch_bounds__(T * B, MB)
   for (int64_t base = (int64_t)blockIdx.x * B; base < a.nlines; base += (int64_t)gridDim.x * B) {
     const int64_t line = base + ly;
     const bool act = line < a.nlines;
-    const float2* src = a.cin + line * a.cpitch;
     float2* dst = reinterpret_cast<float2*>(a.rout) + line * L;
     const int jt = opaque_tid_x();
-    // the L + 1 inputs as the pairs (X[k], X[L-k]), k <= L/2 (k = 0 pairs
-    // X[0] with X[L]): every load issued before the first shared store, so
-    // that they are all in flight together
-    constexpr int NP = (L / 2) / T + 1;
-    float2 xa[NP], xb[NP];
+    // the L + 1 inputs as the pairs (X[k], X[L-k]), k < L/2 (k = 0 pairs X[0]
+    // with X[L]), and X[L/2]: every load issued before the first shared store,
+    // so that they are all in flight together
+    const RealGroup<L, T> g(ly, jt);
+    const int64_t gline = base + g.first;
+    float2 xa[g.NPAIR], xb[g.NPAIR];
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      const int k = jt + i * T;
-      const bool ok = act && k <= L / 2;
-      xa[i] = ok ? src[k] : make_float2(0.f, 0.f);
-      xb[i] = ok ? src[L - k] : make_float2(0.f, 0.f);
+    for (int n = 0; n < g.NPAIR; ++n) {
+      int i, k;
+      const bool ok = g.pair(n, i, k) && gline + i < a.nlines;
+      const float2* row = a.cin + (gline + i) * a.cpitch;
+      xa[n] = ok ? row[k] : make_float2(0.f, 0.f);
+      xb[n] = ok ? row[L - k] : make_float2(0.f, 0.f);
     }
+    const bool mid = g.lane < g.LINES;
+    float2 xmid = make_float2(0.f, 0.f);
+    if (mid && gline + g.lane < a.nlines) xmid = a.cin[(gline + g.lane) * a.cpitch + L / 2];
     line_sync<T>();  // the previous line group is done with sl
     // Z[k] and Z[L-k] of each pair: with e, q = i w^-k d of k, Z[k] = e + q
     // and (w^-(L-k) = -w^k, the roles of X[k], X[L-k] swap) Z[L-k] =
     // conj(e - q); stored conjugated (backward = conj o forward o conj).
     // The imaginary parts of X[0] and X[L] are ignored; k = L/2 is its own
     // partner.
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      const int k = jt + i * T;
-      if (k <= L / 2) {
-        float2 xk = xa[i], xm = xb[i];
-        if (k == 0) {
-          xk.y = 0.f;
-          xm.y = 0.f;
-        }
-        const float2 e = make_float2(xk.x + xm.x, xk.y - xm.y);      // X[k] + conj X[L-k]
-        const float2 d = make_float2(xk.x - xm.x, xk.y + xm.y);      // X[k] - conj X[L-k]
-        const float2 w = __ldg(&a.tw2[k]);
-        const float2 od = cmul(make_float2(w.x, -w.y), d);           // w^-k d
-        const float2 qv = make_float2(-od.y, od.x);                  // i w^-k d
-        sl[padp<P>(k)] = make_float2(e.x + qv.x, -(e.y + qv.y));     // conj Z[k]
-        if (k > 0 && 2 * k != L) sl[padp<P>(L - k)] = make_float2(e.x - qv.x, e.y - qv.y);  // conj Z[L-k]
+    auto store = [&](int i, int k, float2 xk, float2 xm) {
+      float2* z = smem + (g.first + i) * LP;
+      if (k == 0) {
+        xk.y = 0.f;
+        xm.y = 0.f;
       }
+      const float2 e = make_float2(xk.x + xm.x, xk.y - xm.y);      // X[k] + conj X[L-k]
+      const float2 d = make_float2(xk.x - xm.x, xk.y + xm.y);      // X[k] - conj X[L-k]
+      const float2 w = __ldg(&a.tw2[k]);
+      const float2 od = cmul(make_float2(w.x, -w.y), d);           // w^-k d
+      const float2 qv = make_float2(-od.y, od.x);                  // i w^-k d
+      z[padp<P>(k)] = make_float2(e.x + qv.x, -(e.y + qv.y));      // conj Z[k]
+      if (k > 0 && 2 * k != L) z[padp<P>(L - k)] = make_float2(e.x - qv.x, e.y - qv.y);  // conj Z[L-k]
+    };
+#pragma unroll
+    for (int n = 0; n < g.NPAIR; ++n) {
+      int i, k;
+      if (g.pair(n, i, k)) store(i, k, xa[n], xb[n]);
     }
+    if (mid) store(g.lane, L / 2, xmid, xmid);
     line_sync<T>();
     float2 v[emax<L, T, Rs...>()];
     static_for<0, NST>([&](auto S) {
@@ -181,7 +233,8 @@ __global__ void __launch_bounds__(T * B, MB)
 #pragma unroll
             for (int r = 0; r < R; ++r) v[q * R + r] = sl[padp<P>(jt + q * T + r * (L / R))];
       }
-      spec_stage<L, T, R, Ns>(v, jt, a.tw);
+      constexpr int OFF = stage_table_off<s, Rs...>();
+      spec_stage<L, T, R, Ns, OFF>(v, jt, OFF < 0 ? a.tw : a.tws);
     });
     constexpr int RL = radix_at<NST - 1, Rs...>();
 #pragma unroll

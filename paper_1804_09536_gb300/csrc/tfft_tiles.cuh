@@ -68,17 +68,53 @@ __device__ __forceinline__ bool bf_exists(int jt, int q) {
   else return jt + q * T < L / R;
 }
 
+// Offset of stage s in a plan's stage table (launch_stage_twiddles): stages
+// 1 .. s - 1 hold (R - 1) Ns entries each.
+template <int S, int... Rs>
+__host__ __device__ constexpr int stage_table_at() {
+  constexpr int r[] = {Rs...};
+  int off = 0, ns = r[0];
+  for (int i = 1; i < S; ++i) {
+    off += (r[i] - 1) * ns;
+    ns *= r[i];
+  }
+  return off;
+}
+
+// Where a contiguous pass reads stage s's twiddles (spec_stage's OFF): the
+// stage table, except for 512 and 1024 in two stages, which are no faster with
+// it (512^3 pass 0.310 ms either way; 1024 x 64 x 1024 165 us from the roots,
+// 172 from the table).  With it: 2048 50 -> 34 us, 240 24.6 -> 22.5 us,
+// Bluestein 333 59 -> 53 us.
+template <int S, int... Rs>
+__host__ __device__ constexpr int stage_table_off() {
+  constexpr int r[] = {Rs...};
+  return r[0] == 32 && sizeof...(Rs) == 2 ? -1 : stage_table_at<S, Rs...>();
+}
+
 // Twiddle (stage span Ns > 1) and size-R butterflies of a thread's work items.
-template <int L, int T, int R, int Ns, int EM>
+// OFF < 0: tw is the table of the L roots; otherwise it is the plan's stage
+// table, whose stage starts at OFF and holds twiddle r of butterflies k = 0 ..
+// Ns - 1 consecutively.  In the contiguous passes a warp's lanes have
+// consecutive k: one line of 16 twiddles per load instead of up to 16 lines
+// (root r k L / (Ns R) lies r k apart), which kept the L1 busier than the data
+// did.
+template <int L, int T, int R, int Ns, int OFF = -1, int EM>
 __device__ __forceinline__ void spec_stage(float2 (&v)[EM], int jt, const float2* __restrict__ tw) {
 #pragma unroll
   for (int q = 0; q < nbf<L, T, R>(); ++q) {
     if (!bf_exists<L, T, R>(jt, q)) continue;
     if constexpr (Ns > 1) {
       const int j = jt + q * T;
-      const int step = (j % Ns) * (L / (Ns * R));
+      if constexpr (OFF >= 0) {
+        const float2* row = tw + OFF + j % Ns;
 #pragma unroll
-      for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], __ldg(&tw[r * step]));
+        for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], __ldg(row + (r - 1) * Ns));
+      } else {
+        const int step = (j % Ns) * (L / (Ns * R));
+#pragma unroll
+        for (int r = 1; r < R; ++r) v[q * R + r] = cmul(v[q * R + r], __ldg(&tw[r * step]));
+      }
     }
     Dft<R>::run(&v[q * R]);
   }
@@ -242,7 +278,8 @@ __device__ __forceinline__ void contig_tile(const ContigArgs& a, int64_t tile, f
 #pragma unroll
           for (int r = 0; r < R; ++r) v[q * R + r] = sl[padp<P>(jt + q * T + r * (L / R))];
     }
-    spec_stage<L, T, R, Ns>(v, jt, a.tw);
+    constexpr int OFF = CG ? -1 : stage_table_off<s, Rs...>();
+    spec_stage<L, T, R, Ns, OFF>(v, jt, OFF < 0 ? a.tw : a.tws);
   });
   constexpr int RL = radix_at<NST - 1, Rs...>();
   const float oscale = contig_scale(a);
@@ -453,10 +490,11 @@ __device__ __forceinline__ void strided_stages(float2 (&v)[emax<L, T, Rs...>()],
 }
 
 // The same for one contiguous line in its padded line slot sl (the
-// contiguous passes' layout), synchronising the line's threads.
+// contiguous passes' layout), synchronising the line's threads; tws: the
+// stage table of these radices.
 template <int L, int T, int... Rs>
 __device__ __forceinline__ void line_stages(float2 (&v)[emax<L, T, Rs...>()], float2* sl, int jt,
-                                            const float2* __restrict__ tw) {
+                                            const float2* __restrict__ tws) {
   constexpr int NST = sizeof...(Rs);
   constexpr int P = pad_every<Rs...>();
   static_for<0, NST>([&](auto S) {
@@ -479,7 +517,7 @@ __device__ __forceinline__ void line_stages(float2 (&v)[emax<L, T, Rs...>()], fl
 #pragma unroll
           for (int r = 0; r < R; ++r) v[q * R + r] = sl[padp<P>(jt + q * T + r * (L / R))];
     }
-    spec_stage<L, T, R, Ns>(v, jt, tw);
+    spec_stage<L, T, R, Ns, stage_table_at<s, Rs...>()>(v, jt, tws);
   });
 }
 
