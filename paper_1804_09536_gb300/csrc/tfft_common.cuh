@@ -31,7 +31,7 @@ struct DevLayout {
   int64_t N[MAXD];
   int64_t Mx[MAXD];
   int64_t rs[MAXD];
-  const int64_t* offset;  // nranks entries (device memory in kernels)
+  const int64_t* offset;  // nranks entries and the total (device memory in kernels)
   int64_t pitch;          // > 0: the innermost axis is stored `pitch` apart (a padded internal layout)
 };
 

@@ -305,6 +305,14 @@ int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st, 
     a.oax1 = oax[1];
     a.on1 = oax[1] >= 0 ? p->cshape[oax[1]] : 1;
     a.W = s.W;
+    if (s.axis == 0 && s.lin == s.lout && s.ncols < 0 && p->st[s.lin].owner[0] < 0 && p->st[s.lin].pitch == 0) {
+      int64_t inner = 0;
+      const LayoutH& L = p->st[s.lin];
+      for (int r = 0; r < L.nranks; ++r)
+        inner = std::max(inner, ((r + 1 < L.nranks ? L.offset[r + 1] : L.total) - L.offset[r]) / s.L);
+      a.merged_blocks = (inner + s.W - 1) / s.W;
+      a.nranks = L.nranks;
+    }
     a.sign = s.sign;
     a.scale = s.scaled ? (float)s.scale_value : 1.0f;
     a.status = reinterpret_cast<int*>(p->d_state);

@@ -143,6 +143,10 @@ struct StridedArgs {
   int oax0, oax1;         // the outer axes (or -1), outer index = g[oax0] * on1 + g[oax1]
   int64_t on1;
   int W;                  // block width (blockDim.x)
+  // > 0: an in-place pass along the leading, uncut axis over every column: the
+  // W-column blocks of the rank with most of them (see merged_tile)
+  int64_t merged_blocks = 0;
+  int nranks = 0;
   int sign;
   float scale;
   int* status;            // device status word

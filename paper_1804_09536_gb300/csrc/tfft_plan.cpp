@@ -71,6 +71,13 @@ void build_layout(tfft_plan p, const int64_t* shape, int stage, LayoutH& L, int6
   L.pitch = pitch;
 }
 
+// The rank offsets of a layout, and its total, as the kernels read them.
+size_t add_offsets(tfft_plan p, const LayoutH& L) {
+  std::vector<int64_t> v = L.offset;
+  v.push_back(L.total);
+  return image_add(p, v.data(), v.size() * sizeof(int64_t));
+}
+
 DevLayout dev_layout(tfft_plan p, const LayoutH& L) {
   DevLayout D;
   D.d = L.d;
@@ -402,7 +409,7 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
     p->st.resize(p->g + 1);
     for (int s = 0; s <= p->g; ++s) {
       build_layout(p, p->cshape, s, p->st[s]);
-      p->st[s].state_off = image_add(p, p->st[s].offset.data(), p->st[s].offset.size() * 8);
+      p->st[s].state_off = add_offsets(p, p->st[s]);
     }
     if (kind == TFFT_R2C) build_layout(p, p->shape, 0, p->real0);
     // per-length FFT plans and twiddle table slots (a plan whose lengths do not

@@ -260,6 +260,7 @@ namespace host {
 // ---- plan state image, layouts, per-length plans (tfft_plan.cpp)
 size_t image_add(tfft_plan p, const void* data, size_t bytes);
 void build_layout(tfft_plan p, const int64_t* shape, int stage, LayoutH& L, int64_t pitch = 0);
+size_t add_offsets(tfft_plan p, const LayoutH& L);
 DevLayout dev_layout(tfft_plan p, const LayoutH& L);
 bool make_axis_plan(int L, bool strided, AxisPlan& best);
 int strided_width(const AxisPlan& ap);

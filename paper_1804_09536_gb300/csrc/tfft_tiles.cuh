@@ -450,7 +450,74 @@ __device__ __forceinline__ void strided_tile(const StridedArgs& a, int64_t tile,
     }
 }
 
-
+// One tile of an in-place pass along the leading axis of a layout that holds
+// it whole (the last pass of every fused forward, the first of a backward).
+// A rank's local array is then L rows of `inner` consecutive elements, all of
+// them columns of independent lines, however many axes and odd extents they
+// come from: the tile is up to W of them at column block `tile` mod
+// a.merged_blocks of rank `tile` / a.merged_blocks, row i of it `inner`
+// elements after row i - 1.  No column blocks, no row tables, no fold: every
+// thread places the tile with one division and two loads, and only a rank's
+// last tile is partial.
+template <int L, int T, int W, bool CHAIN, int... Rs>
+__device__ __forceinline__ void merged_tile(const StridedArgs& a, uint32_t tile, float2* smem, int cx, int jt) {
+  constexpr int NST = sizeof...(Rs);
+  const bool inv = a.sign > 0;
+  const uint32_t rank = tile / (uint32_t)a.merged_blocks;
+  const int c0 = (int)(tile - rank * (uint32_t)a.merged_blocks) * W;
+  const int o0 = (int)__ldg(&a.lin.offset[rank]);
+  const int inner = ((int)__ldg(&a.lin.offset[rank + 1]) - o0) / L;
+  if constexpr (CHAIN)
+    if (tile == blockIdx.x) chain_wait();
+  if (c0 >= inner) return;  // a rank with fewer blocks than the widest (the whole CTA leaves)
+  const bool act = c0 + cx < inner;
+  // lanes past the last column load it again and store nothing
+  const int at = o0 + (act ? c0 + cx : inner - 1);
+  const float2* src = a.in + at;
+  float2 v[emax<L, T, Rs...>()];
+  static_for<0, NST>([&](auto S) {
+    constexpr int s = decltype(S)::value;
+    constexpr int R = radix_at<s, Rs...>();
+    constexpr int Ns = span_at<s, Rs...>();
+    if constexpr (s == 0) {
+#pragma unroll
+      for (int q = 0; q < nbf<L, T, R>(); ++q)
+        if (bf_exists<L, T, R>(jt, q))
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            float2 x = src[(jt + q * T) * inner + r * (L / R) * inner];
+            if (inv) x.y = -x.y;
+            v[q * R + r] = x;
+          }
+    } else {
+      constexpr int Rp = radix_at<s - 1, Rs...>();
+      constexpr int Nsp = Ns / Rp;
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < nbf<L, T, Rp>(); ++q)
+        if (bf_exists<L, T, Rp>(jt, q))
+#pragma unroll
+          for (int r = 0; r < Rp; ++r)
+            smem[stockham_out_index(jt + q * T, Nsp, Rp, r) * W + cx] = v[q * Rp + r];
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < nbf<L, T, R>(); ++q)
+        if (bf_exists<L, T, R>(jt, q))
+#pragma unroll
+          for (int r = 0; r < R; ++r) v[q * R + r] = smem[(jt + q * T + r * (L / R)) * W + cx];
+    }
+    spec_stage<L, T, R, Ns>(v, jt, a.tw);
+  });
+  constexpr int RL = radix_at<NST - 1, Rs...>();
+  const float sc = a.scale, scy = inv ? -a.scale : a.scale;
+  float2* dst = a.out + at;
+#pragma unroll
+  for (int q = 0; q < nbf<L, T, RL>(); ++q)
+    if (act && bf_exists<L, T, RL>(jt, q))
+#pragma unroll
+      for (int r = 0; r < RL; ++r)
+        dst[(jt + q * T) * inner + r * (L / RL) * inner] = make_float2(v[q * RL + r].x * sc, v[q * RL + r].y * scy);
+}
 
 // ------------------------------------------------------------ stages only
 

@@ -405,7 +405,7 @@ bool plan_padding(tfft_plan p) {
     p->st.pop_back();
     return false;
   }
-  p->st[idx].state_off = image_add(p, p->st[idx].offset.data(), p->st[idx].offset.size() * 8);
+  p->st[idx].state_off = add_offsets(p, p->st[idx]);
   p->pad_stage = idx;
   p->pad_lead = lead;
   p->win_c0 = c0;
