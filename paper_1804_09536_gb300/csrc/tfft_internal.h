@@ -287,7 +287,6 @@ struct BoxArgs {
   float2* out;
   const CopyTask* tasks;
   int64_t ntasks;
-  int vec2;  // every offset, stride and row length is even: 16-byte copies
 };
 
 cudaError_t launch_contig(const ContigArgs& a, cudaStream_t s);
