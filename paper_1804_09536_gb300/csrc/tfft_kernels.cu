@@ -441,7 +441,8 @@ __global__ void __launch_bounds__(512) k_blue_strided(const StridedArgs a, const
 // threads in order, whatever the row length (an element's row is one multiply
 // by the reciprocal of the row length; a task has at most 2^16 of them), and
 // every thread keeps U of them in flight before it stores them.  A task whose
-// offsets, strides and row length are all even moves 16 bytes at a time.
+// ends are 16-byte aligned and whose strides and row length are even moves 16
+// bytes at a time.
 //
 // The copy is bound by loads in flight: with rows dealt to power-of-two lane
 // groups (31 of 64 lanes idle on 33-element rows) and 64 registers, four CTAs
@@ -478,11 +479,16 @@ __global__ void __launch_bounds__(256, 8) k_boxcopy(const BoxArgs a) {
   const CopyTask t = a.tasks[blockIdx.x];
   if (t.nrows <= 0 || t.rowlen <= 0) return;
   const uint32_t total = (uint32_t)t.nrows * (uint32_t)t.rowlen;
-  if ((t.src | t.dst | t.ss | t.ds | (int64_t)t.rowlen) & 1)
-    copy_task<float2, 4>(a.in + t.src, a.out + t.dst, t.ss, t.ds, (uint32_t)t.rowlen, total);
+  const float2* src = a.in + t.src;
+  float2* dst = a.out + t.dst;
+  // the base pointers count too: the second workspace buffer of an unfused
+  // transform starts one stage buffer in, 8-byte aligned when that is odd
+  if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) ||
+      ((t.ss | t.ds | (int64_t)t.rowlen) & 1))
+    copy_task<float2, 4>(src, dst, t.ss, t.ds, (uint32_t)t.rowlen, total);
   else
-    copy_task<float4, 4>(reinterpret_cast<const float4*>(a.in + t.src), reinterpret_cast<float4*>(a.out + t.dst),
-                         t.ss / 2, t.ds / 2, (uint32_t)t.rowlen / 2, total / 2);
+    copy_task<float4, 4>(reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst), t.ss / 2, t.ds / 2,
+                         (uint32_t)t.rowlen / 2, total / 2);
 }
 
 // ------------------------------------------------------------ twiddles
