@@ -31,6 +31,7 @@ struct DevLayout {
   int64_t N[MAXD];
   int64_t Mx[MAXD];
   int64_t rs[MAXD];
+  int32_t q[MAXD], r[MAXD];  // N / Mx and N mod Mx
   const int64_t* offset;  // nranks entries and the total (device memory in kernels)
   int64_t pitch;          // > 0: the innermost axis is stored `pitch` apart (a padded internal layout)
 };

@@ -85,6 +85,8 @@ DevLayout dev_layout(tfft_plan p, const LayoutH& L) {
     D.N[m] = L.N[m];
     D.Mx[m] = L.owner[m] >= 0 ? p->grid[L.owner[m]] : 1;
     D.rs[m] = L.owner[m] >= 0 ? p->rstride[L.owner[m]] : 0;
+    D.q[m] = (int32_t)(D.N[m] / D.Mx[m]);
+    D.r[m] = (int32_t)(D.N[m] % D.Mx[m]);
   }
   D.offset = reinterpret_cast<const int64_t*>(p->d_state + L.state_off);
   D.pitch = L.pitch;

@@ -59,6 +59,12 @@ __global__ void __launch_bounds__(W * T, MB) k_strided_merged(const StridedArgs 
     merged_tile<L, T, W, CHAIN, Rs...>(a, tile, smem, threadIdx.x, opaque_tid_y());
 }
 
+template <int L, int T, int W, int MB, int... Rs>
+__global__ void __launch_bounds__(W * T, MB) k_strided_gather(const StridedArgs a) {
+  extern __shared__ float2 smem[];
+  gather_tiles<L, T, W, Rs...>(a, smem);
+}
+
 // the kernel's shared-memory limit raised to 227 KB, once per device
 #define TFFT_ALLOW_SMEM(kernel)                          \
   static PerDevice<cudaError_t> attr_cache;              \
@@ -106,6 +112,20 @@ cudaError_t run_strided_tiles(K kern, const StridedArgs& a, size_t smem, int64_t
 
 template <int L, int T, int W, int MB, bool CHAIN, int... Rs>
 cudaError_t run_strided(const StridedArgs& a, cudaStream_t s) {
+  // Gathering passes, where the two placing warps are a small part of the CTA
+  // (256 threads: 400^3 0.244 -> 0.224 ms per pass, 128^4 0.70 -> 0.674, 256 x
+  // 256 x 240 forward + inverse 261 -> 253 us; but 180 x 200 x 240, whose 200
+  // runs five warps, 149 -> 154) or the pass is chained, when its set-up runs
+  // before the wait (100 x 150 x 180 63.0 -> 60.3, 96 x 200 x 96 40.7 -> 39.2;
+  // shorter lines gain nothing: 60 x 72 x 100 19.2 -> 19.5).
+  if constexpr (!CHAIN && L <= 1024)
+    if (a.merged_blocks == 0 && (W * T >= 256 || (a.chained && L >= 96)) && a.lin.Mx[a.axis] <= kGatherParts &&
+        a.lout.Mx[a.axis] <= kGatherParts) {
+      static PerDevice<cudaError_t> attr_cache;
+      static PerDevice<int64_t> slots_cache;
+      return run_strided_tiles<L, T, W>(k_strided_gather<L, T, W, MB, Rs...>, a, gather_smem<L, W>(),
+                                        a.nouter * a.ncolblocks, a.chained, s, attr_cache, slots_cache);
+    }
   if constexpr (!CHAIN && chainable(L))
     if (a.chained) return run_strided<L, T, W, MB, true, Rs...>(a, s);
   const int chained = CHAIN ? a.chained : 0;

@@ -519,6 +519,184 @@ __device__ __forceinline__ void merged_tile(const StridedArgs& a, uint32_t tile,
         dst[(jt + q * T) * inner + r * (L / RL) * inner] = make_float2(v[q * RL + r].x * sc, v[q * RL + r].y * scy);
 }
 
+// ------------------------------------------------------------ gathering passes
+//
+// Passes whose layouts cut the FFT axis (the axis d - 2 pass of a fused
+// transform gathers its lines from one cut and scatters them to another): row
+// i of a tile lies at part[c] + l prod for its part c and index l there.
+// Where strided_tile folds a tile in two threads and builds both row tables
+// behind three barriers before its first load, here the next tile is placed,
+// one lane per part, and both its tables are built between the exchanges of
+// the current one; one barrier per tile is left beside the exchanges'.
+
+// Where a tile lies in one layout: the rank part and the index before (head)
+// and after (tail, rows `prod` apart) the FFT axis, in 32 bits (every offset of
+// a specialised pass fits).
+struct TilePlace {
+  uint32_t base, head, prod, tail;
+  int2 blk;
+  __device__ __forceinline__ TilePlace(const StridedArgs& a, const DevLayout& lay, uint32_t tile) {
+    const uint32_t o = tile / (uint32_t)a.ncolblocks;
+    blk = a.colblocks[tile - o * (uint32_t)a.ncolblocks];
+    uint32_t go0 = o, go1 = 0;
+    if (a.oax1 >= 0) {
+      go0 = o / (uint32_t)a.on1;
+      go1 = o - go0 * (uint32_t)a.on1;
+    }
+    base = head = tail = 0;
+    prod = 1;
+#pragma unroll
+    for (int m = 0; m < MAXD; ++m) {
+      if (m >= lay.d || m == a.axis) continue;
+      const uint32_t g = (m == a.d - 1) ? (uint32_t)blk.x : (m == a.oax0) ? go0 : (m == a.oax1) ? go1 : 0;
+      uint32_t local = g, n = (uint32_t)lay.q[m];
+      if (lay.Mx[m] > 1) {  // inverse of Eq. decompose
+        const uint32_t r = (uint32_t)lay.r[m], big = r * (n + 1);
+        uint32_t c;
+        if (g < big) {
+          c = g / (n + 1);
+          local = g - c * (n + 1);
+          n += 1;
+        } else {
+          c = (g - big) / n;
+          local = g - big - c * n;
+          c += r;
+        }
+        base += c * (uint32_t)lay.rs[m];
+      }
+      if (m == lay.d - 1 && lay.pitch > 0) n = (uint32_t)lay.pitch;  // the innermost axis' storage extent
+      if (m < a.axis) {
+        head = head * n + local;
+      } else {
+        tail = tail * n + local;
+        prod *= n;
+      }
+    }
+  }
+};
+
+// Parts of each layout a CTA can hold (of each of two tiles).
+constexpr int kGatherParts = 64;
+
+struct GatherShared {
+  int part[2][2][kGatherParts];  // offset of index 0 of every part: slot, side (input, output)
+  int prod[2][2];
+  int2 blk[2];
+};
+
+template <int L, int W>
+__host__ __device__ constexpr size_t gather_smem() {
+  return (size_t)L * W * sizeof(float2) + 4 * (size_t)L * sizeof(int) + sizeof(GatherShared);
+}
+
+// Places tile `tile` in slot p: threads 0 .. 31 the parts of the input layout
+// (one each, in rounds), 32 .. 63 those of the output layout.
+__device__ __forceinline__ void gather_place(const StridedArgs& a, uint32_t tile, GatherShared* gs, int p, int tid) {
+  if (tid >= 64) return;
+  const int side = tid >> 5;
+  const DevLayout& lay = side ? a.lout : a.lin;
+  const TilePlace t(a, lay, tile);
+  const uint32_t q = (uint32_t)lay.q[a.axis], r = (uint32_t)lay.r[a.axis];
+  for (uint32_t c = (uint32_t)tid & 31; c < (uint32_t)lay.Mx[a.axis]; c += 32)
+    gs->part[p][side][c] = (int)((uint32_t)lay.offset[t.base + c * (uint32_t)lay.rs[a.axis]] +
+                                 t.head * (q + (c < r ? 1 : 0)) * t.prod + t.tail);
+  if ((tid & 31) == 0) gs->prod[p][side] = (int)t.prod;
+  if (tid == 0) gs->blk[p] = t.blk;
+}
+
+// All tiles of a CTA.
+template <int L, int T, int W, int... Rs>
+__device__ __forceinline__ void gather_tiles(const StridedArgs& a, float2* smem) {
+  constexpr int NST = sizeof...(Rs);
+  static_assert(W * T >= 64 && NST >= 2, "two placing warps, one exchange at least");
+  int* rin = reinterpret_cast<int*>(smem + L * W);
+  int* rout = rin + L;
+  uint32_t* rp = reinterpret_cast<uint32_t*>(rout + L);  // part and index of every row of both layouts, for the CTA's life
+  GatherShared* gs = reinterpret_cast<GatherShared*>(rp + 2 * L);
+  const int cx = threadIdx.x;
+  const int tid = threadIdx.y * W + cx;
+  const bool inv = a.sign > 0;
+  const uint32_t ntiles = (uint32_t)(a.nouter * a.ncolblocks);
+  if (a.chained) chain_next();
+  for (uint32_t i = (uint32_t)tid; i < 2 * L; i += W * T) {
+    const DevLayout& lay = i < L ? a.lin : a.lout;
+    const uint32_t q = (uint32_t)lay.q[a.axis], r = (uint32_t)lay.r[a.axis], big = r * (q + 1);
+    const uint32_t row = i < L ? i : i - L;
+    const uint32_t c = row < big ? row / (q + 1) : r + (row - big) / q;
+    rp[i] = (c << 16) | (row - c * q - (c < r ? c : r));
+  }
+  gather_place(a, blockIdx.x, gs, 0, tid);
+  __syncthreads();
+  auto build_rows = [&](int* rows, int side, int p) {
+    const int prod = gs->prod[p][side];
+    const int* part = gs->part[p][side];
+    for (int i = tid; i < L; i += W * T) {
+      const uint32_t cl = rp[side * L + i];
+      rows[i] = part[cl >> 16] + (int)(cl & 0xFFFF) * prod;
+    }
+  };
+  build_rows(rin, 0, 0);
+  if (a.chained) chain_wait();
+  int p = 0;
+  for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x, p ^= 1) {
+    __syncthreads();  // the tile's input rows are complete
+    const int jt = opaque_tid_y();
+    const int2 blk = gs->blk[p];
+    const bool act = cx < blk.y;
+    const bool more = tile + gridDim.x < ntiles;
+    float2 v[emax<L, T, Rs...>()];
+    static_for<0, NST>([&](auto S) {
+      constexpr int s = decltype(S)::value;
+      constexpr int R = radix_at<s, Rs...>();
+      constexpr int Ns = span_at<s, Rs...>();
+      if constexpr (s == 0) {
+#pragma unroll
+        for (int q = 0; q < nbf<L, T, R>(); ++q)
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            const int pos = jt + q * T + r * (L / R);
+            float2 x = (act && bf_exists<L, T, R>(jt, q)) ? a.in[rin[pos] + cx] : make_float2(0.f, 0.f);
+            if (inv) x.y = -x.y;
+            v[q * R + r] = x;
+          }
+      } else {
+        constexpr int Rp = radix_at<s - 1, Rs...>();
+        constexpr int Nsp = Ns / Rp;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < nbf<L, T, Rp>(); ++q)
+          if (bf_exists<L, T, Rp>(jt, q))
+#pragma unroll
+            for (int r = 0; r < Rp; ++r) smem[stockham_out_index(jt + q * T, Nsp, Rp, r) * W + cx] = v[q * Rp + r];
+        if constexpr (s == 1) {
+          // every thread is past the previous tile's stores and this one's
+          // loads: both tables and the other slot are free
+          build_rows(rout, 1, p);
+          if (more) gather_place(a, tile + gridDim.x, gs, p ^ 1, tid);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < nbf<L, T, R>(); ++q)
+          if (bf_exists<L, T, R>(jt, q))
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[q * R + r] = smem[(jt + q * T + r * (L / R)) * W + cx];
+        if constexpr (s == 1)
+          if (more) build_rows(rin, 0, p ^ 1);
+      }
+      spec_stage<L, T, R, Ns>(v, jt, a.tw);
+    });
+    constexpr int RL = radix_at<NST - 1, Rs...>();
+#pragma unroll
+    for (int q = 0; q < nbf<L, T, RL>(); ++q)
+#pragma unroll
+      for (int r = 0; r < RL; ++r) {
+        float2 x = cscale(v[q * RL + r], a.scale);
+        if (inv) x.y = -x.y;
+        if (act && bf_exists<L, T, RL>(jt, q)) a.out[rout[jt + q * T + r * (L / RL)] + cx] = x;
+      }
+  }
+}
+
 // ------------------------------------------------------------ stages only
 
 // The Stockham stages of a length-L FFT on the values a thread holds for

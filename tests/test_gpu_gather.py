@@ -1,0 +1,28 @@
+"""GPU parity of the gathering passes over the number of parts (needs a GPU): one round of placing
+lanes, two, the most a CTA holds, and more (the row-table pass), with empty and uneven parts."""
+import numpy as np
+import pytest
+
+from oracle import redistribute as R
+from paper_1804_09536_gb300 import inputs
+from gpu_util import RTOL_FP32, bits, rel_l2, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape,grid", [((70, 256, 24), (32,)), ((70, 256, 17), (40,)), ((70, 256, 24), (64,)),
+                                        ((90, 256, 24), (80,)), ((20, 400, 33), (24,)),   # empty parts of axis 0
+                                        ((40, 128, 130), (5, 7)), ((12, 11, 128, 60), (2, 3, 4))])
+def test_parts(cuda_device, shape, grid):
+    from paper_1804_09536_gb300.plan import Plan
+    g = len(grid)
+    x = inputs.uniform_complex(shape, seed=len(shape)).numpy()
+    b0 = R.scatter(x, grid, 0)
+    p = Plan(shape, grid, device=cuda_device, tma=False)
+    y = p.forward(to_dev(b0, cuda_device))
+    yu = p.forward(to_dev(b0, cuda_device), mode="unfused")
+    back = p.inverse(y.clone())
+    want = R.scatter(np.fft.fftn(x.astype(np.complex128)) / x.size, grid, g)
+    assert rel_l2(y.cpu().numpy(), want) <= RTOL_FP32
+    assert rel_l2(back.cpu().numpy(), b0) <= RTOL_FP32
+    assert np.array_equal(bits(y), bits(yu))
