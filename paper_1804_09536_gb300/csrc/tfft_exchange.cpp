@@ -199,6 +199,8 @@ BoxList add_box_list(tfft_plan p, const std::vector<BoxDesc>& boxes) {
     box_tasks(b, tasks);
     L.elems += b.ext[0] * b.ext[1] * b.ext[2] * b.ext[3];
   }
+  for (const CopyTask& t : tasks)
+    if ((t.src | t.dst | t.ss | t.ds | (int64_t)t.rowlen) & 1) L.vec2 = 0;
   L.ntasks = (int64_t)tasks.size();
   L.off = image_add(p, tasks.data(), tasks.size() * sizeof(CopyTask));
   return L;
@@ -312,6 +314,7 @@ Step box_step(const BoxList& L) {
   s.inplace_ok = false;
   s.box_off = L.off;
   s.ntasks = L.ntasks;
+  s.vec2 = L.vec2;
   s.box_elems = L.elems;
   return s;
 }

@@ -402,6 +402,7 @@ int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st, 
     a.out = out;
     a.tasks = reinterpret_cast<const CopyTask*>(p->d_state + s.box_off);
     a.ntasks = s.ntasks;
+    a.vec2 = s.vec2;
     e = launch_boxcopy(a, st);
   }
   if (e != cudaSuccess) return cuda_fail(e, "kernel launch");

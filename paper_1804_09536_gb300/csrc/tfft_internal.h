@@ -287,6 +287,9 @@ struct BoxArgs {
   float2* out;
   const CopyTask* tasks;
   int64_t ntasks;
+  // every offset, stride and row length is even: 16-byte copies (an odd number
+  // of elements has an odd row, so the buffers' starts are aligned then too)
+  int vec2;
 };
 
 cudaError_t launch_contig(const ContigArgs& a, cudaStream_t s);

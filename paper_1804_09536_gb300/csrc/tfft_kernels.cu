@@ -437,58 +437,79 @@ __global__ void __launch_bounds__(512) k_blue_strided(const StridedArgs a, const
 
 // ------------------------------------------------------------ box copy
 
-// One CTA per copy task.  The task's nrows x rowlen elements are dealt to the
-// threads in order, whatever the row length (an element's row is one multiply
-// by the reciprocal of the row length; a task has at most 2^16 of them), and
-// every thread keeps U of them in flight before it stores them.  A task whose
-// ends are 16-byte aligned and whose strides and row length are even moves 16
-// bytes at a time.
-//
-// The copy is bound by loads in flight: with rows dealt to power-of-two lane
-// groups (31 of 64 lanes idle on 33-element rows) and 64 registers, four CTAs
-// per SM, the 512^3 half spectrum's exchanges on 4 x 8 (rows of 32 and 33
-// complex) ran at 4.9 and 4.6 TB/s along axes 2 <-> 1; now 6.4 and 5.4 (219 ->
-// 169 and 235 -> 201 us; six CTAs per SM 187 and 210, eight loads in flight at
-// four CTAs 205 and 221).
+// One CTA per copy task.  The task's rows are spread over the CTA in slots of
+// `lpr` lanes (the smallest power of two covering the row, at most 256), and
+// every thread keeps U rows' loads in flight before it stores them; no
+// division per row or element.  T is float4 (pairs of complex64) when every
+// offset, stride and row length of the launch is even, else float2.
 template <class T, int U>
-__device__ __forceinline__ void copy_task(const T* __restrict__ src, T* __restrict__ dst, int64_t ss, int64_t ds,
-                                          uint32_t rowlen, uint32_t total) {
-  const uint32_t recip = rowlen > 1 ? 0xFFFFFFFFu / rowlen + 1 : 0;
-  for (uint32_t e0 = threadIdx.x; e0 < total; e0 += 256 * U) {
-    T v[U];
+__global__ void __launch_bounds__(256) k_boxcopy_rows(const BoxArgs a) {
+  constexpr int K = sizeof(T) / sizeof(float2);
+  const CopyTask* tp = a.tasks + blockIdx.x;
+  const int nrows = tp->nrows;
+  const int rowlen = tp->rowlen / K;  // in copy units
+  if (nrows <= 0 || rowlen <= 0) return;
+  const T* src = reinterpret_cast<const T*>(a.in + tp->src);
+  T* dst = reinterpret_cast<T*>(a.out + tp->dst);
+  const int64_t ss = tp->ss / K, ds = tp->ds / K;
+  const int lpr = rowlen >= 256 ? 256 : (rowlen <= 1 ? 1 : 1 << (32 - __clz(rowlen - 1)));
+  const int slots = 256 / lpr;
+  const int lane = threadIdx.x % lpr, slot = threadIdx.x / lpr;
+  for (int r0 = slot; r0 < nrows; r0 += slots * U) {
+    for (int c = lane; c < rowlen; c += lpr) {
+      T v[U];
 #pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const uint32_t e = e0 + 256 * k;
-      if (e < total) {
-        const uint32_t r = recip ? __umulhi(e, recip) : e;
-        v[k] = src[r * ss + (e - r * rowlen)];
+      for (int k = 0; k < U; ++k) {
+        const int r = r0 + k * slots;
+        if (r < nrows) v[k] = src[r * ss + c];
       }
-    }
 #pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const uint32_t e = e0 + 256 * k;
-      if (e < total) {
-        const uint32_t r = recip ? __umulhi(e, recip) : e;
-        dst[r * ds + (e - r * rowlen)] = v[k];
+      for (int k = 0; k < U; ++k) {
+        const int r = r0 + k * slots;
+        if (r < nrows) dst[r * ds + c] = v[k];
       }
     }
   }
 }
 
-__global__ void __launch_bounds__(256, 8) k_boxcopy(const BoxArgs a) {
+// The same for launches with odd rows that fill the chip more than once: the
+// task's nrows x rowlen elements are dealt to the threads in order, whatever
+// the row length (an element's row is one multiply by the reciprocal of the
+// row length; a task has at most 2^14 of them), at 32 registers and eight CTAs
+// per SM.  The copy is bound by loads in flight: in power-of-two lane groups
+// (31 of 64 lanes idle on 33-element rows) at four CTAs per SM the 512^3 half
+// spectrum's exchanges on 4 x 8 (rows of 32 and 33 complex) took 219 and 235
+// us along axes 2 <-> 1, now 169 and 201 (six CTAs 187 and 210; eight loads in
+// flight at four CTAs 205 and 221).  Even launches, whose 16-byte copies need
+// fewer, and launches of one wave, bound by latency, are faster by rows (128^3
+// on 2 x 4 both exchanges 15.5 against 16.2 us, 64^3 7.9 against 9.0).
+template <int U>
+__global__ void __launch_bounds__(256, 8) k_boxcopy_dense(const BoxArgs a) {
   const CopyTask t = a.tasks[blockIdx.x];
   if (t.nrows <= 0 || t.rowlen <= 0) return;
-  const uint32_t total = (uint32_t)t.nrows * (uint32_t)t.rowlen;
-  const float2* src = a.in + t.src;
-  float2* dst = a.out + t.dst;
-  // the base pointers count too: the second workspace buffer of an unfused
-  // transform starts one stage buffer in, 8-byte aligned when that is odd
-  if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) ||
-      ((t.ss | t.ds | (int64_t)t.rowlen) & 1))
-    copy_task<float2, 4>(src, dst, t.ss, t.ds, (uint32_t)t.rowlen, total);
-  else
-    copy_task<float4, 4>(reinterpret_cast<const float4*>(src), reinterpret_cast<float4*>(dst), t.ss / 2, t.ds / 2,
-                         (uint32_t)t.rowlen / 2, total / 2);
+  const uint32_t rowlen = (uint32_t)t.rowlen, total = (uint32_t)t.nrows * rowlen;
+  const uint32_t recip = rowlen > 1 ? 0xFFFFFFFFu / rowlen + 1 : 0;
+  const float2* __restrict__ src = a.in + t.src;
+  float2* __restrict__ dst = a.out + t.dst;
+  for (uint32_t e0 = threadIdx.x; e0 < total; e0 += 256 * U) {
+    float2 v[U];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const uint32_t e = e0 + 256 * k;
+      if (e < total) {
+        const uint32_t r = recip ? __umulhi(e, recip) : e;
+        v[k] = src[r * t.ss + (e - r * rowlen)];
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const uint32_t e = e0 + 256 * k;
+      if (e < total) {
+        const uint32_t r = recip ? __umulhi(e, recip) : e;
+        dst[r * t.ds + (e - r * rowlen)] = v[k];
+      }
+    }
+  }
 }
 
 // ------------------------------------------------------------ twiddles
@@ -653,7 +674,12 @@ cudaError_t launch_strided_blue(const StridedArgs& a, const BlueArgs& b, cudaStr
 cudaError_t launch_boxcopy(const BoxArgs& a, cudaStream_t s) {
   if (a.ntasks <= 0) return cudaSuccess;
   if (a.ntasks > 0x7fffffff) return cudaErrorInvalidConfiguration;
-  k_boxcopy<<<(unsigned)a.ntasks, 256, 0, s>>>(a);
+  if (a.vec2)
+    k_boxcopy_rows<float4, 4><<<(unsigned)a.ntasks, 256, 0, s>>>(a);
+  else if (a.ntasks <= 4 * (int64_t)device_sm_count())
+    k_boxcopy_rows<float2, 4><<<(unsigned)a.ntasks, 256, 0, s>>>(a);
+  else
+    k_boxcopy_dense<4><<<(unsigned)a.ntasks, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -92,6 +92,7 @@ struct Step {
   // box copies: the copy tasks of the step's box list
   size_t box_off = 0;
   int64_t ntasks = 0;
+  int vec2 = 0;
   int64_t box_elems = 0;
   // TMA-staged strided pass: variant, its column blocks and the tile
   // geometry of the input and output layouts
@@ -134,10 +135,11 @@ struct ExchangeBoxes {  // one adjacent-stage exchange
 };
 
 // A box list as the copy kernel runs it: offset of its task table in the
-// plan state, task count, elements copied.
+// plan state, task count, whether 16-byte copies apply, elements copied.
 struct BoxList {
   size_t off = 0;
   int64_t ntasks = 0;
+  int vec2 = 1;
   int64_t elems = 0;
 };
 
