@@ -117,7 +117,7 @@ def load(path: str = LIB_PATH):
 
 def call(name, *args):
     """Call an ABI function; raise TfftError on a non-zero status."""
-    lib = load()
+    lib = _lib or load()
     rc = getattr(lib, name)(*args)
     if rc != 0:
         msg = lib.tfft_last_error()

@@ -447,15 +447,13 @@ int execute_impl(tfft_plan p, int key, int sign, int mode, const void* in, void*
     const char* b = static_cast<const char*>(out);
     if (a < b + out_bytes && b < a + in_bytes) return fail(TFFT_EINVAL, "in and out overlap");
   }
-  std::vector<Step> steps = p->steps[{key, mode}];
+  const std::vector<Step>& plain = p->steps[{key, mode}];
+  int last = -1;
   if (coef || factor != 1.0) {  // device coefficient and host factor go on the last transform pass
-    int k = (int)steps.size() - 1;
-    while (k >= 0 && steps[k].kind == S_BOX) --k;
-    if (k < 0 || steps[k].kind != S_CONTIG)
+    last = (int)plain.size() - 1;
+    while (last >= 0 && plain[last].kind == S_BOX) --last;
+    if (last < 0 || plain[last].kind != S_CONTIG)
       return fail(TFFT_EUNSUPPORTED, "a device coefficient needs a contiguous last pass");
-    steps[k].coef = coef;
-    steps[k].scale_value = (steps[k].scaled ? steps[k].scale_value : 1.0) * factor;
-    steps[k].scaled = true;
   }
   void* w0 = nullptr;
   void* w1 = nullptr;
@@ -492,13 +490,24 @@ int execute_impl(tfft_plan p, int key, int sign, int mode, const void* in, void*
       if (a < b + sizes[k] && b < a + wb) return fail(TFFT_EINVAL, "work overlaps in or out");
     }
   }
-  assign_buffers(steps, destroy);
-  if (!p->events.empty() && p->events.size() < steps.size() + 1)
+  if (!p->events.empty() && p->events.size() < plain.size() + 1)
     return fail(TFFT_EINVAL, "fewer launch events than launches + 1");
+  // this call's steps: made only when they are launched or captured, not when
+  // their graph is replayed
+  auto make_steps = [&] {
+    std::vector<Step> steps = plain;
+    if (last >= 0) {
+      steps[last].coef = coef;
+      steps[last].scale_value = (steps[last].scaled ? steps[last].scale_value : 1.0) * factor;
+      steps[last].scaled = true;
+    }
+    assign_buffers(steps, destroy);
+    return steps;
+  };
   void* bufs[4] = {const_cast<void*>(in), out, w0, w1};
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (!allow_graph || !p->events.empty() || (p->flags & TFFT_NO_GRAPH)) return run_steps(p, steps, bufs, st);
-  return run_steps_cached(p, tfft_plan_s::GraphKey{key, mode, in, out, w0, w1, coef, factor, p->wait_limit}, steps,
+  if (!allow_graph || !p->events.empty() || (p->flags & TFFT_NO_GRAPH)) return run_steps(p, make_steps(), bufs, st);
+  return run_steps_cached(p, tfft_plan_s::GraphKey{key, mode, in, out, w0, w1, coef, factor, p->wait_limit}, make_steps,
                           bufs, st);
 }
 
@@ -507,14 +516,14 @@ int execute_impl(tfft_plan p, int key, int sign, int mode, const void* in, void*
 // capture stream and instantiates them, that call and later ones launch the
 // graph on `st`.  A stream already being captured by the caller, or a failed
 // capture, launches directly.
-int run_steps_cached(tfft_plan p, const tfft_plan_s::GraphKey& k, const std::vector<Step>& steps, void* const* bufs,
+int run_steps_cached(tfft_plan p, const tfft_plan_s::GraphKey& k, const std::function<std::vector<Step>()>& make_steps, void* const* bufs,
                      cudaStream_t st) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
     cudaGetLastError();
-    return run_steps(p, steps, bufs, st);
+    return run_steps(p, make_steps(), bufs, st);
   }
-  if (cs != cudaStreamCaptureStatusNone) return run_steps(p, steps, bufs, st);
+  if (cs != cudaStreamCaptureStatusNone) return run_steps(p, make_steps(), bufs, st);
   std::lock_guard<std::mutex> lock(p->graph_mutex);
   const int dev = current_device();
   if (p->graph_device >= 0 && p->graph_device != dev) p->release_graphs();
@@ -547,7 +556,7 @@ int run_steps_cached(tfft_plan p, const tfft_plan_s::GraphKey& k, const std::vec
     cudaError_t ce = cudaStreamBeginCapture(p->capture_stream, cudaStreamCaptureModeRelaxed);
     int rc = TFFT_OK;
     if (ce == cudaSuccess) {
-      rc = run_steps(p, steps, bufs, p->capture_stream);
+      rc = run_steps(p, make_steps(), bufs, p->capture_stream);
       ce = cudaStreamEndCapture(p->capture_stream, &g);
     }
     if (rc == TFFT_OK && ce == cudaSuccess && g) ce = cudaGraphInstantiate(&e.exec, g, 0);
@@ -557,10 +566,10 @@ int run_steps_cached(tfft_plan p, const tfft_plan_s::GraphKey& k, const std::vec
       cudaGetLastError();
       e.exec = nullptr;
       e.calls = -(1 << 30);
-      return run_steps(p, steps, bufs, st);
+      return run_steps(p, make_steps(), bufs, st);
     }
   }
-  if (!e.exec) return run_steps(p, steps, bufs, st);
+  if (!e.exec) return run_steps(p, make_steps(), bufs, st);
   cudaError_t ce = cudaGraphLaunch(e.exec, st);
   if (ce != cudaSuccess) return cuda_fail(ce, "cudaGraphLaunch");
   return TFFT_OK;

@@ -302,7 +302,8 @@ void assign_buffers(std::vector<Step>& v, bool destroy_input);
 int launch_step(tfft_plan p, const Step& s, void* const* bufs, cudaStream_t st, int chained = 0);
 int chain_flags(tfft_plan p, size_t k);
 int run_steps(tfft_plan p, const std::vector<Step>& steps, void* const* bufs, cudaStream_t st);
-int run_steps_cached(tfft_plan p, const tfft_plan_s::GraphKey& k, const std::vector<Step>& steps, void* const* bufs,
+int run_steps_cached(tfft_plan p, const tfft_plan_s::GraphKey& k,
+                     const std::function<std::vector<Step>()>& make_steps, void* const* bufs,
                      cudaStream_t st);
 int execute_impl(tfft_plan p, int key, int sign, int mode, const void* in, void* out, void* work,
                  size_t work_bytes, void* stream, const double* coef = nullptr, double factor = 1.0,

@@ -136,12 +136,12 @@ class Plan:
         return torch.empty(self.stage_elems(stage, real), dtype=dt, device=self.device)
 
     def workspace(self, mode: str = "fused", keep_input: bool = True) -> torch.Tensor | None:
-        nb = self.workspace_bytes(mode, keep_input)
-        if nb == 0:
-            return None
         key = (mode, keep_input)
         w = self._work.get(key)
-        if w is None or w.numel() < nb:
+        if w is None:  # its size is fixed when the plan is created
+            nb = self.workspace_bytes(mode, keep_input)
+            if nb == 0:
+                return None
             w = torch.empty(nb, dtype=torch.uint8, device=self.device)
             self._work[key] = w
         return w
