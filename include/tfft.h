@@ -303,7 +303,8 @@ int tfft_plan_num_launches(tfft_plan plan, int sign, int mode, int *nlaunches);
  * (a column window of a real-to-complex pencil plan; the next launch is the
  * plain kernel over the remaining columns, and each reports the bytes of
  * its own columns), ..._tc_bf16x3 / _tc_fp16x3 (tensor-core stage),
- * fft_strided_bluestein_L<n>, fft_r2c_L<n> / fft_c2r_L<n>, box_copy.
+ * fft_strided_bluestein_L<n> / fft_strided_rader_L<n> (lengths without compiled
+ * factors), fft_r2c_L<n> / fft_c2r_L<n>, box_copy.
  */
 int tfft_plan_launch_info(tfft_plan plan, int sign, int mode, int index, char *name,
                           int name_len, int64_t *bytes);

@@ -42,6 +42,22 @@ int blue_spec_length(int N) {
   return best;
 }
 
+bool rader_plan(int N, int& tile_width) {
+#define X(MM, T, W, ...)  \
+  if (N == MM + 1) {      \
+    tile_width = W;       \
+    return true;          \
+  }
+  TFFT_RADER_STRIDED(X)
+#undef X
+  return false;
+}
+
+cudaError_t launch_strided_rader(const StridedArgs& a, const BlueArgs& b, cudaStream_t s) {
+  return spec::with_part((b.N - 1) % spec::kSpecParts,
+                         [&](auto p) { return blue::rader_strided_part<decltype(p)::value>(a, b, s); });
+}
+
 cudaError_t launch_contig_blue_spec(const ContigArgs& a, const BlueArgs& b, cudaStream_t s) {
   return spec::with_part(b.M % spec::kSpecParts,
                          [&](auto p) { return blue::blue_contig_part<decltype(p)::value>(a, b, s); });

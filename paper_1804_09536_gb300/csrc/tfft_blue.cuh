@@ -225,6 +225,149 @@ __global__ void __launch_bounds__(W * T, MB) k_blue_strided_spec(const StridedAr
   }
 }
 
+// ------------------------------------------------------------ prime lengths
+//
+// Rader's form for a prime N whose M = N - 1 has compiled stages: with a
+// primitive root g, X[g^-k] = x[0] + sum_q x[g^q] w^(g^(q - k)) is a cyclic
+// convolution of length N - 1 itself, against Bluestein's 2N - 1 or more, and
+// the permutations cost nothing where rows are read and written through
+// tables: position q of the tile is row g^q on the way in and row g^-q on the
+// way out.  Y = FFT_M(x[g^q]) bhat with bhat = FFT_M(w^(g^-q)) / M; x[0] added
+// to Y[0] reaches every output of the inverse, and X[0] is x[0] plus bin 0 of
+// the first FFT, both in the hands of one thread.
+template <int M, int W>
+__host__ __device__ constexpr size_t rader_strided_smem() {
+  return (size_t)M * W * sizeof(float2) + 2 * (size_t)(M + 1) * sizeof(int) + sizeof(TileShared) +
+         2 * (size_t)(M + 1) * sizeof(uint32_t) + 16;
+}
+
+template <int M, int T, int W, int MB, int... Rs>
+__global__ void __launch_bounds__(W * T, MB) k_rader_strided(const StridedArgs a, const BlueArgs b) {
+  constexpr int NST = sizeof...(Rs), N = M + 1;
+  constexpr int R0 = radix_at<0, Rs...>(), RL = radix_at<NST - 1, Rs...>();
+  using Rev = typename Reverse<Radices<>, Rs...>::type;
+  static_assert(W * T > 32, "the two layouts' folds are computed by threads 0 and 32");
+  extern __shared__ float2 smem[];
+  TileShared* ts = reinterpret_cast<TileShared*>(smem + M * W);
+  int* rin = reinterpret_cast<int*>(ts + 1);
+  int* rout = rin + N;
+  uint32_t* rp = reinterpret_cast<uint32_t*>(rout + N);
+  const int cx = threadIdx.x;
+  const int tid = threadIdx.y * W + cx;
+  const bool inv = a.sign > 0;
+  const int64_t ntiles = a.nouter * a.ncolblocks;
+  chain_next();
+  // part and index of every position's row in both layouts, once per CTA:
+  // position i < M is row perm[i], position M is row 0
+  for (int i = tid; i < 2 * N; i += W * T) {
+    const bool out = i >= N;
+    const int pos = out ? i - N : i;
+    const int row = pos < M ? __ldg(&b.perm[out ? M + pos : pos]) : 0;
+    const int64_t NN = out ? a.lout.N[a.axis] : a.lin.N[a.axis];
+    const int64_t MM = out ? a.lout.Mx[a.axis] : a.lin.Mx[a.axis];
+    int64_t c = 0, l = row, n = NN;
+    if (MM > 1) locate(NN, MM, row, c, l, n);
+    rp[i] = ((uint32_t)c << 16) | (uint32_t)l;
+  }
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    __syncthreads();  // the previous tile is done with the tables, the scalars and smem
+    if (tid == 0) {
+      const StridedTilePos tp(a, tile);
+      tile_fold(a, a.lin, tp, ts, 0);
+      ts->blk = tp.blk;
+    } else if (tid == 32) {
+      const StridedTilePos tp(a, tile);
+      tile_fold(a, a.lout, tp, ts, 1);
+    }
+    __syncthreads();
+    for (int i = tid; i < 2 * N; i += W * T) {
+      const bool out = i >= N;
+      const int64_t c = rp[i] >> 16, l = rp[i] & 0xFFFF;
+      if (out)
+        rout[i - N] = row_offset(a.lout, a.axis, ts, 1, c, l);
+      else
+        rin[i] = row_offset(a.lin, a.axis, ts, 0, c, l);
+    }
+    __syncthreads();
+    const int2 blk = ts->blk;
+    const bool act = cx < blk.y;
+    const int jt = opaque_tid_y();
+    if (tile == blockIdx.x) chain_wait();
+    float2 v[emax<M, T, Rs...>()];
+#pragma unroll
+    for (int q = 0; q < nbf<M, T, R0>(); ++q)
+#pragma unroll
+      for (int r = 0; r < R0; ++r) {
+        float2 x = make_float2(0.f, 0.f);
+        if (act && bf_exists<M, T, R0>(jt, q)) x = a.in[rin[jt + q * T + r * (M / R0)] + cx];
+        if (inv) x.y = -x.y;
+        v[q * R0 + r] = x;
+      }
+    // x[0], for the thread that holds bin 0 of the convolution
+    float2 x0 = make_float2(0.f, 0.f);
+    if (act && jt == 0) {
+      x0 = a.in[rin[M] + cx];
+      if (inv) x0.y = -x0.y;
+    }
+    stages<M, T, W, true>(Radices<Rs...>{}, v, smem, cx, jt, b.twr);
+    const float2 sum = v[0];
+    apply_filter<M, T, RL>(v, jt, b.rhat);
+    if (jt == 0) {
+      v[0] = cadd(v[0], conjf2(x0));
+      if (act) {
+        float2 y = cscale(cadd(sum, x0), a.scale);
+        if (inv) y.y = -y.y;
+        a.out[rout[M] + cx] = y;
+      }
+    }
+    stages<M, T, W, true>(Rev{}, v, smem, cx, jt, b.twr);
+#pragma unroll
+    for (int q = 0; q < nbf<M, T, R0>(); ++q)
+#pragma unroll
+      for (int r = 0; r < R0; ++r)
+        if (act && bf_exists<M, T, R0>(jt, q)) {
+          float2 y = cscale(conjf2(v[q * R0 + r]), a.scale);
+          if (inv) y.y = -y.y;
+          a.out[rout[jt + q * T + r * (M / R0)] + cx] = y;
+        }
+  }
+}
+
+// Compiled M = N - 1: threads per column, tile width, CTAs per SM, radices.
+#define TFFT_RADER_STRIDED(X) \
+  X(28, 2, 32, 12, 14, 2)     \
+  X(30, 2, 32, 12, 15, 2)     \
+  X(36, 3, 32, 8, 6, 6)       \
+  X(40, 2, 32, 10, 2, 20)     \
+  X(42, 3, 32, 8, 14, 3)      \
+  X(60, 4, 32, 6, 15, 4)      \
+  X(70, 5, 32, 4, 14, 5)      \
+  X(72, 6, 16, 8, 6, 12)      \
+  X(96, 4, 32, 4, 8, 12)      \
+  X(100, 5, 32, 4, 20, 5)     \
+  X(108, 6, 16, 6, 18, 6)     \
+  X(112, 8, 16, 6, 8, 14)     \
+  X(126, 7, 16, 4, 21, 6)     \
+  X(150, 5, 16, 6, 5, 30)     \
+  X(162, 9, 16, 4, 9, 18)     \
+  X(180, 15, 16, 3, 15, 12)   \
+  X(192, 16, 16, 3, 16, 12)   \
+  X(196, 14, 16, 3, 14, 14)   \
+  X(210, 15, 16, 3, 15, 14)   \
+  X(240, 16, 16, 3, 16, 15)   \
+  X(250, 13, 16, 2, 25, 10)   \
+  X(256, 16, 16, 3, 16, 16)   \
+  X(270, 18, 16, 2, 15, 18)   \
+  X(280, 10, 16, 3, 28, 10)   \
+  X(336, 14, 16, 2, 28, 12)   \
+  X(378, 14, 16, 2, 14, 27)   \
+  X(400, 20, 16, 2, 20, 20)   \
+  X(420, 21, 16, 1, 20, 21)   \
+  X(432, 24, 16, 1, 24, 18)   \
+  X(448, 32, 16, 1, 8, 14, 4) \
+  X(486, 54, 16, 1, 9, 6, 9)  \
+  X(490, 35, 16, 1, 14, 5, 7)
+
 // Compiled convolution lengths.  Contiguous: M, threads per line, lines per
 // CTA, CTAs per SM, radices; strided: M, threads per column, tile width, CTAs
 // per SM, radices.  The passes are bound by instruction issue, so a length
@@ -311,9 +454,29 @@ cudaError_t run_blue_strided(const StridedArgs& a, const BlueArgs& b, cudaStream
   return launch_chained(k_blue_strided_spec<M, T, W, MB, Rs...>, dim3((unsigned)grid), dim3(W, T), smem, s, a.chained, a,
                         b);
 }
+
+template <int M, int T, int W, int MB, int... Rs>
+cudaError_t run_rader_strided(const StridedArgs& a, const BlueArgs& b, cudaStream_t s) {
+  TFFT_ALLOW_SMEM((k_rader_strided<M, T, W, MB, Rs...>));
+  if (attr != cudaSuccess) return attr;
+  if (a.W != W || b.N != M + 1) return cudaErrorInvalidValue;
+  constexpr size_t smem = rader_strided_smem<M, W>();
+  static PerDevice<int64_t> slots_cache;
+  const int64_t slots = slots_cache.get(current_device(), [&] {
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rader_strided<M, T, W, MB, Rs...>, W * T, smem);
+    return (int64_t)device_sm_count() * (per_sm > 0 ? per_sm : 1);
+  });
+  int64_t grid = a.nouter * a.ncolblocks;
+  if (grid > slots) grid = slots;
+  if (grid < 1) return cudaSuccess;
+  return launch_chained(k_rader_strided<M, T, W, MB, Rs...>, dim3((unsigned)grid), dim3(W, T), smem, s, a.chained, a, b);
+}
 #undef TFFT_ALLOW_SMEM
 
 // compiled with the specialised passes' parts (tfft_spec_part.cu)
+template <int P>
+cudaError_t rader_strided_part(const StridedArgs& a, const BlueArgs& b, cudaStream_t s);
 template <int P>
 cudaError_t blue_contig_part(const ContigArgs& a, const BlueArgs& b, cudaStream_t s);
 template <int P>

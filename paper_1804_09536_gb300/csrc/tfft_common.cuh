@@ -439,6 +439,7 @@ struct AxisPlan {
   int width;       // lines per CTA (contiguous) or tile width W (strided)
   int radix[MAXSTAGES];
   int blue_m;      // > 0: length without a 2/3/5 plan, done by Bluestein with this convolution length
+  int rader;       // 1: strided passes of a prime length with a compiled Rader convolution
   int blue_spec;   // 1: that convolution length has compile-time specialised kernels (width is theirs)
 };
 

@@ -52,6 +52,12 @@ struct BlueArgs {
   int N, M;
   AxisPlan apm;          // length-M FFT plan (shared-memory stages)
   const float2* twm;     // the M roots exp(-2 pi i m / M)
+  // strided passes of a prime N by Rader's convolution of length N - 1
+  // (AxisPlan::rader): its roots, the rows g^q then g^-q (q < N - 1) and the
+  // filter spectrum
+  const float2* twr;
+  const int* perm;
+  const float2* rhat;
   const float2* tws_f;   // stage tables of the contiguous pass's two FFTs
   const float2* tws_r;
   const float2* chirp;   // N values exp(-i pi (n^2 mod 2N) / N)
@@ -306,6 +312,9 @@ void blue_spec_radices(int M, int& nst, int* radix);
 int blue_spec_length(int N);
 cudaError_t launch_contig_blue_spec(const ContigArgs& a, const BlueArgs& b, cudaStream_t s);
 cudaError_t launch_strided_blue_spec(const StridedArgs& a, const BlueArgs& b, cudaStream_t s);
+// Rader passes of a prime length N: whether N has one and its tile width.
+bool rader_plan(int N, int& tile_width);
+cudaError_t launch_strided_rader(const StridedArgs& a, const BlueArgs& b, cudaStream_t s);
 cudaError_t launch_twiddles(float2* tw, int L, cudaStream_t s);
 // Stage table of a length-L plan (L entries reserved): for every stage after
 // the first (span Ns, radix R) the twiddles exp(-2 pi i r k / (Ns R)), r = 1 ..

@@ -218,6 +218,46 @@ bool is_smooth_235(int64_t n) {
   return n == 1;
 }
 
+// Tables of Rader's convolution for a prime N: the rows g^q and g^-q (g the
+// smallest primitive root) and the filter spectrum FFT_M(exp(-2 pi i g^-q / N))
+// / M, M = N - 1, evaluated in double and rounded once.
+void make_rader(tfft_plan p, int N, tfft_plan_s::BlueH& h) {
+  const int M = N - 1;
+  const double pi = 3.14159265358979323846;
+  int g = 2;
+  std::vector<int> pw(M);
+  for (;; ++g) {  // g is primitive when its powers do not return to 1 early
+    int64_t v = 1;
+    int q = 0;
+    for (; q < M; ++q) {
+      if (q > 0 && v == 1) break;
+      pw[q] = (int)v;
+      v = v * g % N;
+    }
+    if (q == M) break;
+  }
+  std::vector<int> perm(2 * M);
+  for (int q = 0; q < M; ++q) {
+    perm[q] = pw[q];
+    perm[M + q] = pw[(M - q) % M];
+  }
+  std::vector<std::complex<double>> w(M), b(M);
+  for (int m = 0; m < M; ++m) {
+    w[m] = std::polar(1.0, -2.0 * pi * (double)m / (double)M);
+    b[m] = std::polar(1.0, -2.0 * pi * (double)perm[M + m] / (double)N);
+  }
+  std::vector<float2> rhat(M);
+  for (int k = 0; k < M; ++k) {
+    std::complex<double> acc = 0.0;
+    for (int m = 0; m < M; ++m) acc += b[m] * w[((int64_t)m * k) % M];
+    acc /= (double)M;
+    rhat[k] = make_float2((float)acc.real(), (float)acc.imag());
+  }
+  h.perm_off = image_add(p, perm.data(), perm.size() * sizeof(int));
+  h.rhat_off = image_add(p, rhat.data(), rhat.size() * sizeof(float2));
+  if (!p->tw_off.count(M)) p->tw_off[M] = image_add(p, nullptr, (size_t)M * sizeof(float2));
+}
+
 // Bluestein plan for a length N without a compiled factorisation: convolution
 // length M = the smallest compiled one >= 2N - 1, or the power of two where
 // the compiled passes do not apply (at most MAXLEN), and the tables,
@@ -277,6 +317,14 @@ bool make_bluestein(tfft_plan p, int N) {
     add_stage_table(p, f);
     add_stage_table(p, std::vector<int>(f.rbegin(), f.rend()));
   }
+  // a prime length whose N - 1 has compiled stages: Rader's convolution in the
+  // strided passes
+  int rader_w = 0;
+  if (aps.blue_spec && rader_plan(N, rader_w)) {
+    make_rader(p, N, h);
+    aps.rader = 1;
+    aps.width = rader_w;
+  }
   p->aplan[N] = ap;
   p->aplan_s[N] = aps;
   p->blue[N] = h;
@@ -303,6 +351,13 @@ BlueArgs blue_args(tfft_plan p, int N) {
   b.apm = h.apm;
   b.twm = reinterpret_cast<const float2*>(p->d_state + p->tw_off.at(h.M));
   b.tws_f = b.tws_r = nullptr;
+  b.twr = b.rhat = nullptr;
+  b.perm = nullptr;
+  if (p->aplan_s.at(N).rader) {
+    b.twr = reinterpret_cast<const float2*>(p->d_state + p->tw_off.at(N - 1));
+    b.perm = reinterpret_cast<const int*>(p->d_state + h.perm_off);
+    b.rhat = reinterpret_cast<const float2*>(p->d_state + h.rhat_off);
+  }
   if (p->aplan.at(N).blue_spec) {
     AxisPlan f{}, r{};
     blue_spec_radices(h.M, f.nst, f.radix);

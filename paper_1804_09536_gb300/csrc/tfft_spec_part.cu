@@ -54,6 +54,17 @@ cudaError_t blue_strided_part(const StridedArgs& a, const BlueArgs& b, cudaStrea
   return cudaErrorInvalidValue;
 }
 
+template <int P>
+cudaError_t rader_strided_part(const StridedArgs& a, const BlueArgs& b, cudaStream_t s) {
+#define X(MM, T, W, MB, ...)                  \
+  if constexpr (MM % spec::kSpecParts == P)   \
+    if (b.N == MM + 1) return run_rader_strided<MM, T, W, MB, __VA_ARGS__>(a, b, s);
+  TFFT_RADER_STRIDED(X)
+#undef X
+  return cudaErrorInvalidValue;
+}
+
+template cudaError_t rader_strided_part<TFFT_SPEC_PART>(const StridedArgs& a, const BlueArgs& b, cudaStream_t s);
 template cudaError_t blue_contig_part<TFFT_SPEC_PART>(const ContigArgs& a, const BlueArgs& b, cudaStream_t s);
 template cudaError_t blue_strided_part<TFFT_SPEC_PART>(const StridedArgs& a, const BlueArgs& b, cudaStream_t s);
 

@@ -1,5 +1,5 @@
-"""GPU parity of the Bluestein passes over their convolution lengths (needs a GPU): the largest and
-the smallest line length of every compiled convolution length, contiguous and strided, on uneven
+"""GPU parity of the Bluestein and Rader passes (needs a GPU): the largest and the smallest line
+length of every compiled convolution length, and every prime with a Rader pass, contiguous and strided, on uneven
 blocks with partial tiles."""
 import os
 import re
@@ -34,7 +34,13 @@ def _lengths():
     return out
 
 
-LENGTHS = _lengths()
+def _rader():
+    text = open(os.path.join(CSRC, "tfft_blue.cuh")).read()
+    body = text[text.index("#define TFFT_RADER_STRIDED"):].split("\n\n")[0]
+    return [int(m) + 1 for m in re.findall(r"X\((\d+),", body)]
+
+
+LENGTHS = sorted(set(_lengths() + _rader()))
 
 
 @pytest.mark.parametrize("N", LENGTHS)
@@ -44,7 +50,7 @@ def test_bluestein_lengths(cuda_device, N):
         x = inputs.uniform_complex(full, seed=N).numpy()
         b0 = R.scatter(x, grid, 0)
         p = Plan(full, grid, device=cuda_device)
-        assert any(n.endswith(f"bluestein_L{N}") for n, _ in p.launch_info(-1))
+        assert any(n.endswith((f"bluestein_L{N}", f"rader_L{N}")) for n, _ in p.launch_info(-1))
         y = p.forward(to_dev(b0, cuda_device))
         yu = p.forward(to_dev(b0, cuda_device), mode="unfused")
         back = p.inverse(y.clone())

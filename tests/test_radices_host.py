@@ -59,7 +59,7 @@ def test_table_rows(name):
 
 
 def test_routes_that_stay():
-    """Lengths refused before are refused, and a prime keeps its Bluestein passes."""
+    """Lengths refused before are refused; a prime whose N - 1 factors takes Rader's strided pass."""
     from paper_1804_09536_gb300 import TfftError
     from paper_1804_09536_gb300.plan import Plan
     for shape, kind in [((2058, 8), "c2c"), ((4097, 8), "c2c"), ((16, 200), "r2c"), ((16, 180), "r2c"), ((16, 84), "r2c")]:
@@ -67,4 +67,4 @@ def test_routes_that_stay():
         with pytest.raises(TfftError):
             p.num_launches(-1)
     names = [n for n, _ in Plan((42, 127, 256), (3, 4), bind=False).launch_info(-1)]
-    assert names == ["fft_contig_L256", "fft_strided_bluestein_L127", "fft_strided_L42"]
+    assert names == ["fft_contig_L256", "fft_strided_rader_L127", "fft_strided_L42"]
