@@ -297,7 +297,10 @@ int tfft_plan_num_launches(tfft_plan plan, int sign, int mode, int *nlaunches);
  * Launch `index` of tfft_execute() in a direction and mode: the kernel's
  * name (NUL-terminated, truncated to name_len) and its algorithmic bytes --
  * one read and one write of every element it moves (complex64), the figure
- * a roofline divides by the launch's duration.  Names: fft_contig_L<n>,
+ * a roofline divides by the launch's duration (as the calls timed with launch
+ * events run; without events a plan of at most 32 MiB per stage buffer chains
+ * its launches and runs plain tiles in place of some TMA-staged ones, with
+ * the same result).  Names: fft_contig_L<n>,
  * fft_strided_L<n> (plain tiles), fft_strided_tma_L<n> (TMA-staged tiles),
  * ..._tma_groups_... (rank groups of an uneven layout), ..._tma_window_...
  * (a column window of a real-to-complex pencil plan; the next launch is the

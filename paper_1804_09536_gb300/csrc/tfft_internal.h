@@ -19,6 +19,7 @@ constexpr int TFFT_DEVICE_ETMEM = 4;     // MMAs still running after the clean-u
 // How a pass is launched in a chain of passes (launch_chained()).
 constexpr int kChainAfter = 1;  // may start before the previous kernel has finished
 constexpr int kChainFirst = 4;  // the first pass of a chain: the next may start before it has finished
+constexpr int kChainPlain = 8;  // plain tiles in place of TMA-staged ones
 constexpr int kChainCarve = 2;  // largest shared-memory carve-out, the same for the whole chain
 
 // Lengths whose passes have a chained variant beside the plain one, which is
