@@ -428,7 +428,9 @@ TFFT_HD int stockham_tw_index(int j, int Ns, int R, int r, int L) {
 
 // FFT plan of one axis length, shared by host planning and device kernels.
 // The radices are also packed 5 bits per stage in `code` so that kernels read
-// stage s's radix with a shift instead of an indexed load.
+// stage s's radix with a shift instead of an indexed load.  The struct goes by
+// value into every kernel, ahead of the geometry and the tensor maps: one more
+// int moved those and cost the TMA-staged passes 0.6 % (512^3 1948 -> 1960 us).
 struct AxisPlan {
   int L;           // transform length
   int E;           // elements per thread (every radix divides E)
@@ -439,8 +441,8 @@ struct AxisPlan {
   int width;       // lines per CTA (contiguous) or tile width W (strided)
   int radix[MAXSTAGES];
   int blue_m;      // > 0: length without a 2/3/5 plan, done by Bluestein with this convolution length
-  int rader;       // 1: strided passes of a prime length with a compiled Rader convolution
-  int blue_spec;   // 1: that convolution length has compile-time specialised kernels (width is theirs)
+  int blue_spec;   // 1: that convolution length has compile-time specialised kernels (width is theirs);
+                   // 2: strided passes of a prime length by Rader's convolution (width is theirs)
 };
 
 TFFT_HD int stage_radix(uint64_t code, int s) { return (int)((code >> (5 * s)) & 31); }

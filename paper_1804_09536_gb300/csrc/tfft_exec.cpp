@@ -652,7 +652,7 @@ int tfft_plan_launch_info(tfft_plan p, int sign, int mode, int index, char* name
            (tma ? "_tma" : "") + (s.kind == S_STRIDED && s.tma_groups && !s.tc ? "_groups" : "") +
            (s.kind == S_STRIDED && s.tma_win ? "_window" : "") +
            (tc ? (p->precision == TFFT_TC_BF16X3 ? "_tc_bf16x3" : "_tc_fp16x3") : "") +
-           (ap.blue_m ? (ap.rader ? "_rader_L" : "_bluestein_L") + std::to_string(ap.L)
+           (ap.blue_m ? (ap.blue_spec == 2 ? "_rader_L" : "_bluestein_L") + std::to_string(ap.L)
                       : ap.spec ? "_L" + std::to_string(ap.L)
                                 : ap.E == 0 ? std::string("_generic") : "_E" + std::to_string(ap.E));
       elems = p->nelems;

@@ -54,7 +54,7 @@ struct BlueArgs {
   AxisPlan apm;          // length-M FFT plan (shared-memory stages)
   const float2* twm;     // the M roots exp(-2 pi i m / M)
   // strided passes of a prime N by Rader's convolution of length N - 1
-  // (AxisPlan::rader): its roots, the rows g^q then g^-q (q < N - 1) and the
+  // (AxisPlan::blue_spec 2): its roots, the rows g^q then g^-q (q < N - 1) and the
   // filter spectrum
   const float2* twr;
   const int* perm;

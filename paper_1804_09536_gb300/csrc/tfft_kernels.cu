@@ -660,7 +660,7 @@ cudaError_t launch_contig_blue(const ContigArgs& a, const BlueArgs& b, cudaStrea
 }
 
 cudaError_t launch_strided_blue(const StridedArgs& a, const BlueArgs& b, cudaStream_t s) {
-  if (a.ap.rader) return launch_strided_rader(a, b, s);
+  if (a.ap.blue_spec == 2) return launch_strided_rader(a, b, s);
   if (a.ap.blue_spec) return launch_strided_blue_spec(a, b, s);
   TFFT_ALLOW_SMEM(k_blue_strided);
   if (attr != cudaSuccess) return attr;

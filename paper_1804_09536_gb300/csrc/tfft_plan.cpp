@@ -322,7 +322,7 @@ bool make_bluestein(tfft_plan p, int N) {
   int rader_w = 0;
   if (aps.blue_spec && rader_plan(N, rader_w)) {
     make_rader(p, N, h);
-    aps.rader = 1;
+    aps.blue_spec = 2;
     aps.width = rader_w;
   }
   p->aplan[N] = ap;
@@ -353,7 +353,7 @@ BlueArgs blue_args(tfft_plan p, int N) {
   b.tws_f = b.tws_r = nullptr;
   b.twr = b.rhat = nullptr;
   b.perm = nullptr;
-  if (p->aplan_s.at(N).rader) {
+  if (p->aplan_s.at(N).blue_spec == 2) {
     b.twr = reinterpret_cast<const float2*>(p->d_state + p->tw_off.at(N - 1));
     b.perm = reinterpret_cast<const int*>(p->d_state + h.perm_off);
     b.rhat = reinterpret_cast<const float2*>(p->d_state + h.rhat_off);

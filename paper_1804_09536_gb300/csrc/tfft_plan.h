@@ -181,7 +181,7 @@ struct tfft_plan_s {
     int M = 0;
     AxisPlan apm{};
     size_t chirp_off = 0, bhat_off = 0;
-    size_t perm_off = 0, rhat_off = 0;  // Rader tables (aplan_s[N].rader)
+    size_t perm_off = 0, rhat_off = 0;  // Rader tables (aplan_s[N].blue_spec == 2)
   };
   std::map<int, BlueH> blue;
   std::map<std::tuple<int, int, int>, std::pair<size_t, int64_t>> colblocks;  // (lin,lout,W)
