@@ -316,12 +316,15 @@ cudaError_t launch_strided_blue_spec(const StridedArgs& a, const BlueArgs& b, cu
 // Rader passes of a prime length N: whether N has one and its tile width.
 bool rader_plan(int N, int& tile_width);
 cudaError_t launch_strided_rader(const StridedArgs& a, const BlueArgs& b, cudaStream_t s);
-cudaError_t launch_twiddles(float2* tw, int L, cudaStream_t s);
-// Stage table of a length-L plan (L entries reserved): for every stage after
-// the first (span Ns, radix R) the twiddles exp(-2 pi i r k / (Ns R)), r = 1 ..
-// R - 1, k = 0 .. Ns - 1, k fastest -- the values of the root table in the
-// order the contiguous passes read them.
-cudaError_t launch_stage_twiddles(float2* tws, int L, int nst, const int* radix, cudaStream_t s);
+// One twiddle table of a plan state: the L roots (nst = 0) or the stage table
+// of a radix sequence, at byte `off` of the state.
+struct TwiddleTable {
+  int64_t off;
+  int L, nst;
+  int radix[MAXSTAGES];
+};
+// Generates them (the descriptors lie in the state) in one launch.
+cudaError_t launch_twiddles(char* state, const TwiddleTable* tables, int ntables, int max_len, cudaStream_t s);
 
 // Batched persistent executor (tfft_batch.cu).  One segment = the tiles of
 // one pass of one transform; items are numbered consecutively over the

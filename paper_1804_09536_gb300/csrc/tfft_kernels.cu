@@ -514,38 +514,31 @@ __global__ void __launch_bounds__(256, 8) k_boxcopy_dense(const BoxArgs a) {
 
 // ------------------------------------------------------------ twiddles
 
-// exp(-2 pi i m / L) for m < L, evaluated in double precision and rounded to
-// float (the only double-precision arithmetic of the path besides the
-// normalisation factor).
-__global__ void k_twiddles(float2* tw, int L) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m < L) {
-    double s, c;
-    sincospi(2.0 * (double)m / (double)L, &s, &c);
-    tw[m] = make_float2((float)c, (float)(-s));
-  }
-}
-
-struct StageRadices {
-  int n, r[MAXSTAGES];
-};
-
-__global__ void k_stage_twiddles(float2* tws, int L, const StageRadices p) {
+// The twiddle tables of a plan state, one per blockIdx.y, evaluated in double
+// precision and rounded to float (the only double-precision arithmetic of the
+// path besides the normalisation factor): the roots exp(-2 pi i m / L), m < L,
+// or a plan's stage table -- for every stage after the first (span Ns, radix
+// R) the roots m = r k L / (Ns R), r = 1 .. R - 1, k = 0 .. Ns - 1, k fastest.
+__global__ void k_twiddles(char* state, const TwiddleTable* tables) {
+  const TwiddleTable& t = tables[blockIdx.y];
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  float2* out = tws + i;
-  int Ns = p.r[0];
-  for (int s = 1; s < p.n; ++s) {
-    const int R = p.r[s], n = (R - 1) * Ns;
-    if (i < n) {
-      const int m = (i / Ns + 1) * (i % Ns) * (L / (Ns * R));
-      double sn, cs;
-      sincospi(2.0 * (double)m / (double)L, &sn, &cs);
-      *out = make_float2((float)cs, (float)(-sn));
-      return;
+  if (i >= t.L) return;
+  float2* out = reinterpret_cast<float2*>(state + t.off) + i;
+  int m = i;
+  if (t.nst > 0) {
+    m = -1;
+    int Ns = t.radix[0];
+    for (int s = 1; s < t.nst && m < 0; ++s) {
+      const int R = t.radix[s], n = (R - 1) * Ns;
+      if (i < n) m = (i / Ns + 1) * (i % Ns) * (t.L / (Ns * R));
+      i -= n;
+      Ns *= R;
     }
-    i -= n;
-    Ns *= R;
+    if (m < 0) return;
   }
+  double sn, cs;
+  sincospi(2.0 * (double)m / (double)t.L, &sn, &cs);
+  *out = make_float2((float)cs, (float)(-sn));
 }
 
 // the kernel's shared-memory limit raised to 227 KB, once per device
@@ -700,16 +693,9 @@ int device_sm_count() {
   });
 }
 
-cudaError_t launch_stage_twiddles(float2* tws, int L, int nst, const int* radix, cudaStream_t s) {
-  StageRadices p = {};
-  p.n = nst;
-  for (int i = 0; i < nst; ++i) p.r[i] = radix[i];
-  k_stage_twiddles<<<(L + 255) / 256, 256, 0, s>>>(tws, L, p);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_twiddles(float2* tw, int L, cudaStream_t s) {
-  k_twiddles<<<(L + 255) / 256, 256, 0, s>>>(tw, L);
+cudaError_t launch_twiddles(char* state, const TwiddleTable* tables, int ntables, int max_len, cudaStream_t s) {
+  if (ntables < 1) return cudaSuccess;
+  k_twiddles<<<dim3((max_len + 255) / 256, ntables), 256, 0, s>>>(state, tables);
   return cudaGetLastError();
 }
 

@@ -552,6 +552,19 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
       for (int s = 0; s <= p->g; ++s)
         for (auto& kv : p->aplan_s) get_colblocks(p, s, s, strided_width(kv.second));
     }
+    std::vector<TwiddleTable> tables;
+    for (auto& kv : p->tw_off) tables.push_back({(int64_t)kv.second, kv.first, 0, {}});
+    for (auto& kv : p->tws_off) {
+      TwiddleTable t{(int64_t)kv.second, 1, (int)kv.first.size(), {}};
+      for (int i = 0; i < t.nst; ++i) {
+        t.radix[i] = kv.first[i];
+        t.L *= kv.first[i];
+      }
+      tables.push_back(t);
+    }
+    for (const TwiddleTable& t : tables) p->max_table = std::max(p->max_table, t.L);
+    p->ntables = (int)tables.size();
+    p->tables_off = image_add(p, tables.data(), tables.size() * sizeof(TwiddleTable));
     p->state_bytes = align_up(p->image.size(), 256);
     p->image.resize(p->state_bytes, 0);
     *plan = p;
@@ -632,17 +645,9 @@ int tfft_plan_bind(tfft_plan p, void* d_state, size_t bytes, void* stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemcpyAsync(d_state, p->image.data(), p->state_bytes, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync (plan state)");
-    for (auto& kv : p->tw_off) {
-      e = launch_twiddles(reinterpret_cast<float2*>(static_cast<char*>(d_state) + kv.second), kv.first, st);
-      if (e != cudaSuccess) return cuda_fail(e, "twiddle generation");
-    }
-    for (auto& kv : p->tws_off) {
-      int L = 1;
-      for (int r : kv.first) L *= r;
-      e = launch_stage_twiddles(reinterpret_cast<float2*>(static_cast<char*>(d_state) + kv.second), L,
-                                (int)kv.first.size(), kv.first.data(), st);
-      if (e != cudaSuccess) return cuda_fail(e, "twiddle generation");
-    }
+    char* base = static_cast<char*>(d_state);
+    e = launch_twiddles(base, reinterpret_cast<const TwiddleTable*>(base + p->tables_off), p->ntables, p->max_table, st);
+    if (e != cudaSuccess) return cuda_fail(e, "twiddle generation");
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize (bind)");
     p->d_state = static_cast<char*>(d_state);

@@ -177,6 +177,8 @@ struct tfft_plan_s {
   std::map<int, AxisPlan> aplan_s; // strided passes
   std::map<int, size_t> tw_off;
   std::map<std::vector<int>, size_t> tws_off;  // stage tables by their radices
+  size_t tables_off = 0;                       // descriptors of both kinds (TwiddleTable) in the state
+  int ntables = 0, max_table = 0;
   struct BlueH {       // Bluestein lengths: convolution plan and the offsets of their tables
     int M = 0;
     AxisPlan apm{};
