@@ -119,12 +119,12 @@ int tfft_decompose(int64_t N, int64_t M, int64_t p, int64_t *n, int64_t *s);
  * TFFT_NORM_BACKWARD, optionally | TFFT_NO_TMA | TFFT_NO_GRAPH.
  * Complex lengths that factor into 2, 3 and 5 (<= 4096), or into 2, 3, 5 and 7
  * (24 .. 1024), run mixed-radix Stockham passes; any other complex length
- * <= 2048 runs Bluestein's convolution form of the DFT (two power-of-two FFTs
- * of length >= 2N - 1 with FP64-built chirp tables) in the same pass
- * structure.  Longer other lengths
- * (and an r2c half-length without a 2/3/5 plan) leave the plan able to
- * redistribute, but its tfft_execute() and tfft_partial() return
- * TFFT_EUNSUPPORTED.
+ * <= 2048 runs Bluestein's convolution form of the DFT (two FFTs of a compiled
+ * length >= 2N - 1 with FP64-built chirp tables) in the same pass structure;
+ * strided passes of 32 primes N from 29 to 491 run Rader's (length N - 1).
+ * Longer other lengths (and an r2c half-length without a compiled real pass)
+ * leave the plan able to redistribute, but its tfft_execute() and
+ * tfft_partial() return TFFT_EUNSUPPORTED.
  * The plan is a host object; destroy it with tfft_plan_destroy().
  */
 int tfft_plan_create(tfft_plan *plan, int ndims, const int64_t *shape, int grid_ndims,
