@@ -26,3 +26,17 @@ def test_parts(cuda_device, shape, grid):
     assert rel_l2(y.cpu().numpy(), want) <= RTOL_FP32
     assert rel_l2(back.cpu().numpy(), b0) <= RTOL_FP32
     assert np.array_equal(bits(y), bits(yu))
+
+
+@pytest.mark.parametrize("shape,grid", [((512, 512, 32), (1, 2)), ((512, 512, 32), (1, 3)),   # three stages
+                                        ((400, 400, 40), (3, 2)), ((384, 384, 48), (1, 3))])
+def test_column_blocks(cuda_device, shape, grid):
+    """Whole and partial column blocks of plans too large to chain their passes."""
+    from paper_1804_09536_gb300.plan import Plan
+    x = inputs.uniform_complex(shape, seed=len(shape)).numpy()
+    b0 = R.scatter(x, grid, 0)
+    p = Plan(shape, grid, device=cuda_device, tma=False)
+    y = p.forward(to_dev(b0, cuda_device))
+    assert rel_l2(y.cpu().numpy(), R.scatter(np.fft.fftn(x.astype(np.complex128)) / x.size, grid, len(grid))) <= RTOL_FP32
+    assert np.array_equal(bits(y), bits(p.forward(to_dev(b0, cuda_device), mode="unfused")))
+    assert rel_l2(p.inverse(y).cpu().numpy(), b0) <= RTOL_FP32
