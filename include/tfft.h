@@ -123,8 +123,9 @@ int tfft_decompose(int64_t N, int64_t M, int64_t p, int64_t *n, int64_t *s);
  * length >= 2N - 1 with FP64-built chirp tables) in the same pass structure;
  * strided passes of 32 primes N from 29 to 491 run Rader's (length N - 1).
  * Longer other lengths (and an r2c half-length without a compiled real pass)
- * leave the plan able to redistribute, but its tfft_execute() and
- * tfft_partial() return TFFT_EUNSUPPORTED.
+ * leave the plan able to redistribute and to run tfft_partial() along its
+ * other axes, but its tfft_execute(), and tfft_partial() along an axis of such
+ * a length, return TFFT_EUNSUPPORTED.
  * The plan is a host object; destroy it with tfft_plan_destroy().
  */
 int tfft_plan_create(tfft_plan *plan, int ndims, const int64_t *shape, int grid_ndims,

@@ -26,8 +26,10 @@ void decompose(int64_t N, int64_t M, int64_t p, int64_t& n, int64_t& s) {
   s = q * p + std::min(r, p);
 }
 
-
+// A block of the plan's state image: a device offset, so only while the plan is
+// created -- the state buffer has the size the image had then.
 size_t image_add(tfft_plan p, const void* data, size_t bytes) {
+  if (p->state_bytes > 0) throw std::logic_error("table added to a plan whose state is already sized");
   const size_t off = align_up(p->image.size(), 256);
   p->image.resize(off + bytes, 0);
   if (data && bytes) std::memcpy(p->image.data() + off, data, bytes);
@@ -548,10 +550,13 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
               }
           p->steps[{kAdjoint, mode}] = v;
         }
-      // column blocks for in-place partial transforms of every stage
-      for (int s = 0; s <= p->g; ++s)
-        for (auto& kv : p->aplan_s) get_colblocks(p, s, s, strided_width(kv.second));
     }
+    // column blocks of the partial transforms: in place along every axis that a
+    // stage holds and whose length has a plan, also where another length of the
+    // plan has none
+    for (int s = 0; s <= p->g; ++s)
+      for (int m = 0; m < ndims - 1; ++m)
+        if (p->st[s].owner[m] < 0 && p->aplan_s.count((int)p->cshape[m])) fft_step(p, m, s, s, TFFT_FORWARD);
     std::vector<TwiddleTable> tables;
     for (auto& kv : p->tw_off) tables.push_back({(int64_t)kv.second, kv.first, 0, {}});
     for (auto& kv : p->tws_off) {

@@ -1,0 +1,127 @@
+"""What the library launches, on a CUDA runtime of host memory (CPU only).
+
+tests/native/fake_cuda.cpp, linked with the library's own objects in place of cudart, runs plans and
+calls as they are and records each launch, so that the tables a kernel would read can be checked
+against the state buffer they have to lie in.
+"""
+import ctypes
+import glob
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+CSRC = os.path.join(ROOT, "paper_1804_09536_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    from paper_1804_09536_gb300 import _lib, build
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None or not os.path.exists("/usr/local/cuda/include/cuda_runtime.h"):
+        pytest.skip("no host C++ compiler or CUDA headers")
+    build.build()
+    d = tmp_path_factory.mktemp("fake")
+    out, script = str(d / "libtfft_fake.so"), d / "exports.map"
+    script.write_text("{ global: tfft_*; fake_*; local: *; };")  # the fake runtime serves these objects alone
+    objs = [os.path.join(build.BUILD, u[1]) for u in build._units()]
+    subprocess.run([cxx, "-O1", "-std=c++17", "-shared", "-fPIC", "-I", CSRC, "-I", "/usr/local/cuda/include",
+                    os.path.join(HERE, "native", "fake_cuda.cpp"), *objs, f"-Wl,--version-script={script}", "-Wl,-z,defs",
+                    "-o", out], check=True)
+    so = ctypes.CDLL(out)
+    for name, args in _lib.SIGNATURES.items():
+        fn = getattr(so, name)
+        fn.argtypes, fn.restype = args, _lib._RESTYPE.get(name, ctypes.c_int)
+    yield so
+    os.remove(out)
+
+
+def _aligned(nbytes):
+    raw = np.zeros(nbytes + 256, np.uint8)
+    off = -raw.ctypes.data % 256
+    return raw[off:off + nbytes]
+
+
+class Fake:
+    """A plan bound to host memory of exactly the state's size."""
+
+    def __init__(self, lib, shape, grid, kind="c2c", precision=0, flags=0):
+        self.lib, self.shape, self.grid, self.h = lib, shape, grid, ctypes.c_void_p()
+        assert lib.tfft_plan_create(ctypes.byref(self.h), len(shape), (ctypes.c_int64 * len(shape))(*shape), len(grid),
+                                    (ctypes.c_int * len(grid))(*grid), int(kind == "r2c"), precision, flags) == 0
+        nb = ctypes.c_size_t()
+        assert lib.tfft_plan_state_bytes(self.h, ctypes.byref(nb)) == 0
+        self.state = _aligned(nb.value)
+        assert lib.tfft_plan_bind(self.h, self.state.ctypes.data, nb.value, None) == 0
+        self.launches()
+
+    def __del__(self):
+        self.lib.tfft_plan_destroy(self.h)
+
+    def launches(self):
+        """(kernel, grid, threads, column block address, their number, merged blocks) since the last call."""
+        buf = ctypes.create_string_buffer(1 << 16)
+        assert self.lib.fake_launches(buf, len(buf)) < len(buf)
+        rows = [r.split("|", 5) for r in buf.value.decode().splitlines()]
+        return [(r[5], *map(int, r[:5])) for r in rows]
+
+    def column_blocks(self, launch):
+        """The column blocks a strided launch reads, which have to lie in the state; None where it reads none."""
+        kernel, _, _, addr, n, merged = launch
+        if "strided" not in kernel or "k_strided_merged" in kernel or "RankGroupTiles" in kernel:
+            return None
+        lo = self.state.ctypes.data
+        assert lo <= addr and addr + 8 * n <= lo + self.state.size, f"{kernel}: column blocks outside the state"
+        return self.state[addr - lo:addr - lo + 8 * n].view(np.int32).reshape(-1, 2)
+
+
+@pytest.mark.parametrize("shape,grid,kind", [((60, 200), (2,), "r2c"), ((20, 200), (2,), "r2c"), ((8, 60, 200), (2,), "r2c"),
+                                             ((22, 18, 200), (2, 2), "r2c"), ((20, 4099), (2,), "c2c"),
+                                             ((20, 4099, 18), (3, 2), "c2c"), ((64, 128, 4160), (2, 2), "c2c"),
+                                             ((96, 64, 4160), (2,), "c2c"), ((18, 4099, 20, 22), (2, 2, 2), "c2c")])
+def test_partial_of_a_plan_that_does_not_transform(lib, shape, grid, kind):
+    """A length without a plan stops the whole transform, not the partial ones along the other axes."""
+    p = Fake(lib, shape, grid, kind)
+    n = ctypes.c_int()
+    assert lib.tfft_plan_num_launches(p.h, -1, 0, ctypes.byref(n)) == 2
+    _partials(lib, p, shape, grid, kind)
+
+
+@pytest.mark.parametrize("shape,grid,kind,precision", [((64, 96, 64), (2, 2), "c2c", 0), ((20, 127, 33), (3, 2), "c2c", 0),
+                                                       ((512, 256, 64), (2,), "c2c", 1), ((256, 512, 128), (2, 2), "c2c", 1),
+                                                       ((60, 64, 128), (2, 2), "r2c", 0), ((20, 96, 18, 22), (2, 2), "c2c", 0),
+                                                       ((384, 30, 17), (), "c2c", 0), ((18, 200), (3,), "c2c", 0)])
+def test_partial_of_a_plan(lib, shape, grid, kind, precision):
+    _partials(lib, Fake(lib, shape, grid, kind, precision), shape, grid, kind)
+
+
+def _partials(lib, p, shape, grid, kind):
+    """Every partial transform along a strided axis reads column blocks of the state: whole columns,
+    each once."""
+    d, g = len(shape), len(grid)
+    columns = shape[-1] // 2 + 1 if kind == "r2c" else shape[-1]
+    x = _aligned(256)  # no kernel runs
+    ran = 0
+    for stage in range(g + 1):
+        cut = [i if i < g - stage else i + 1 for i in range(g)]
+        for axis in range(d - 1):
+            for sign in (-1, 1):
+                rc = lib.tfft_partial(p.h, stage, axis, sign, x.ctypes.data, None)
+                launched = p.launches()
+                if axis in cut or shape[axis] == 4099:
+                    assert rc != 0 and not launched
+                    continue
+                assert rc == 0 and len(launched) == 1
+                ran += 1
+                blocks = p.column_blocks(launched[0])
+                if blocks is not None:
+                    at = 0
+                    for c, w in blocks:
+                        assert c == at and w > 0
+                        at += w
+                    assert at == columns
+    assert ran > 0
