@@ -46,3 +46,23 @@ def test_chained_equals_unchained(cuda_device, shape, grid, kind, graphs):
     assert p.device_status() == 0
     for k, (w, g) in enumerate(zip(want, got)):
         assert np.array_equal(bits(w), bits(g)), k
+
+
+@pytest.mark.parametrize("shape,grid", [((64, 64, 64), (2, 2)), ((96, 96, 96), (2, 2)), ((128, 128, 128), (2, 4)),
+                                        ((256, 32, 256), (2, 2))])
+def test_tma_tiles_of_small_plans(cuda_device, shape, grid):
+    """The TMA-staged tiles that small plans run only when timed: the bits of a plan without TMA."""
+    from paper_1804_09536_gb300.plan import Plan
+    pt, pp = Plan(shape, grid, device=cuda_device), Plan(shape, grid, device=cuda_device, tma=False)
+    gen = torch.Generator(device="cpu").manual_seed(4)
+    x = torch.view_as_complex(torch.randn(pt.stage_elems(0), 2, generator=gen)).to(cuda_device)
+    for sign in (-1, 1):
+        assert any("_tma_" in n for n, _ in pt.launch_info(sign))
+        evs = [torch.cuda.Event(enable_timing=True) for _ in range(pt.num_launches(sign) + 1)]
+        pt.set_launch_events(evs)
+        got = (pt.forward if sign < 0 else pt.inverse)(x)
+        pt.set_launch_events([])
+        want = (pp.forward if sign < 0 else pp.inverse)(x.clone())
+        torch.cuda.synchronize()
+        assert np.array_equal(bits(got), bits(want))
+    assert pt.device_status() == 0

@@ -69,6 +69,27 @@ class Fake:
         rows = [r.split("|", 5) for r in buf.value.decode().splitlines()]
         return [(r[5], *map(int, r[:5])) for r in rows]
 
+    def execute(self, sign=-1, events=False):
+        """The launches of one call on distinct buffers (no kernel runs)."""
+        n, nb = ctypes.c_int(), ctypes.c_size_t()
+        assert self.lib.tfft_plan_num_launches(self.h, sign, 0, ctypes.byref(n)) == 0
+        ev = (ctypes.c_void_p * (n.value + 1))(*[256] * (n.value + 1))
+        assert self.lib.tfft_plan_set_launch_events(self.h, ev, n.value + 1 if events else 0) == 0
+        assert self.lib.tfft_plan_workspace_bytes(self.h, 0, 1, ctypes.byref(nb)) == 0
+        at = 1 << 40  # addresses only
+        assert self.lib.tfft_execute(self.h, sign, 0, at, 2 * at, 3 * at, nb.value, None) == 0
+        return self.launches()
+
+    def names(self, sign=-1):
+        n, b = ctypes.c_int(), ctypes.c_int64()
+        assert self.lib.tfft_plan_num_launches(self.h, sign, 0, ctypes.byref(n)) == 0
+        out = []
+        for k in range(n.value):
+            buf = ctypes.create_string_buffer(64)
+            assert self.lib.tfft_plan_launch_info(self.h, sign, 0, k, buf, 64, ctypes.byref(b)) == 0
+            out.append(buf.value.decode())
+        return out
+
     def column_blocks(self, launch):
         """The column blocks a strided launch reads, which have to lie in the state; None where it reads none."""
         kernel, _, _, addr, n, merged = launch
@@ -125,3 +146,24 @@ def _partials(lib, p, shape, grid, kind):
                         at += w
                     assert at == columns
     assert ran > 0
+
+
+def test_smoke_reaches_a_tma_staged_pass(lib):
+    """The second case of smoke() launches the TMA kernel, not only a plan that names it."""
+    import __graft_entry__ as entry
+    p = Fake(lib, entry.TMA_SHAPE, entry.TMA_GRID)
+    assert "fft_strided_tma_L512" in p.names()
+    assert [k for k, *_ in p.execute() if "k_strided_tma<512" in k]
+
+
+@pytest.mark.parametrize("shape,grid", [((64, 64, 64), (2, 2)), ((96, 96, 96), (2, 2)), ((128, 128, 128), (2, 4)),
+                                        ((32, 64, 128), (2, 2)), ((32, 512, 64), (2, 2)), ((256, 128, 256), (2, 4)),
+                                        ((60, 64, 100), (2, 3))])
+def test_timed_launches_are_the_named_ones(lib, shape, grid):
+    """A call with launch events runs the kernels launch_info() names, TMA-staged ones where it says so."""
+    p = Fake(lib, shape, grid)
+    for sign in (-1, 1):
+        for name, (kernel, *_) in zip(p.names(sign), p.execute(sign, events=True)):
+            assert ("_tma_" in name) == ("k_strided_tma<" in kernel), (name, kernel)
+            assert ("_groups" in name) == ("RankGroupTiles" in kernel), (name, kernel)
+            assert ("contig" in name) == ("contig" in kernel), (name, kernel)
