@@ -106,9 +106,10 @@ bool encode_stage_map(tfft_plan p, const TmaGeo& G, int axis, int W, const void*
   return r == CUDA_SUCCESS;
 }
 
-// Tile width (and optionally threads per column) requested for the strided
-// TMA pass of length L by the environment, TFFT_TMA_W="512:8:16,256:32"
-// (TFFT_TC_W for the tensor-core passes; used when tuning); 0 when not given.
+// Tile width requested for the strided TMA pass of length L by the environment,
+// TFFT_TMA_W="512:8:16,256:32" (length:width, optionally :elements per thread,
+// returned as threads per column; TFFT_TC_W for the tensor-core passes; used
+// when tuning); 0 when not given.
 int tuned_width(int L, int* T, const char* var) {
   if (T) *T = 0;
   const char* env = std::getenv(var);
@@ -121,7 +122,10 @@ int tuned_width(int L, int* T, const char* var) {
     size_t colon = item.find(':');
     if (colon != std::string::npos && std::atoi(item.substr(0, colon).c_str()) == L) {
       size_t colon2 = item.find(':', colon + 1);
-      if (T && colon2 != std::string::npos) *T = std::atoi(item.substr(colon2 + 1).c_str());
+      if (T && colon2 != std::string::npos) {
+        const int E = std::atoi(item.substr(colon2 + 1).c_str());
+        *T = E > 0 ? (L + E - 1) / E : 0;
+      }
       return std::atoi(item.substr(colon + 1).c_str());
     }
     if (comma == std::string::npos) break;

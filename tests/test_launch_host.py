@@ -167,3 +167,13 @@ def test_timed_launches_are_the_named_ones(lib, shape, grid):
             assert ("_tma_" in name) == ("k_strided_tma<" in kernel), (name, kernel)
             assert ("_groups" in name) == ("RankGroupTiles" in kernel), (name, kernel)
             assert ("contig" in name) == ("contig" in kernel), (name, kernel)
+
+
+@pytest.mark.parametrize("ask,threads", [("512:16", 16), ("512:16:32", 16), ("512:16:16", 32), ("256:16", 16),
+                                         ("512:16:24", 16)])  # 24 is not compiled: the default
+def test_tuning_variable(lib, monkeypatch, ask, threads):
+    """TFFT_TMA_W="length:width:elements per thread" picks the TMA-staged variant of a length."""
+    monkeypatch.setenv("TFFT_TMA_W", ask)
+    p = Fake(lib, (32, 512, 64), (2, 2))
+    kernels = [k for k, *_ in p.execute() if "k_strided_tma<512" in k]
+    assert kernels and f"k_strided_tma<512, {threads}, 16," in kernels[0], kernels
