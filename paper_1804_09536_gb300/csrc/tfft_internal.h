@@ -28,6 +28,14 @@ constexpr int kChainCarve = 2;  // largest shared-memory carve-out, the same for
 // 5331).
 constexpr bool chainable(int L) { return L <= 256; }
 
+// Whether the contiguous and real passes of a row (its number of stages and
+// first radix) read their twiddles from the row's stage table; the others read
+// the table of the roots and get no stage table: 512 (32.16) and 1024 (32.32)
+// are no faster with one (512^3 pass 0.310 ms either way; 1024 x 64 x 1024 165
+// us from the roots, 172 from the table).  With it: 2048 50 -> 34 us, 240 24.6
+// -> 22.5 us, Bluestein 333 59 -> 53 us.
+constexpr bool reads_stage_table(int nst, int first_radix) { return nst != 2 || first_radix != 32; }
+
 // Batched 1-D FFT of contiguous lines (the axis held whole and innermost,
 // Eq. pencil0 / slab0): line l of the buffer is elements [l L, (l + 1) L).
 struct ContigArgs {

@@ -340,6 +340,12 @@ void add_stage_table(tfft_plan p, std::vector<int> radices) {
   if (!p->tws_off.count(radices)) p->tws_off[radices] = image_add(p, nullptr, (size_t)L * sizeof(float2));
 }
 
+// The stage table of a contiguous or real row, where its kernel reads one.
+void add_row_table(tfft_plan p, const AxisPlan& ap) {
+  if (reads_stage_table(ap.nst, ap.radix[0])) add_stage_table(p, std::vector<int>(ap.radix, ap.radix + ap.nst));
+}
+
+// The stage table of a plan's radices, NULL where it has none.
 const float2* stage_table(tfft_plan p, const AxisPlan& ap) {
   auto it = p->tws_off.find(std::vector<int>(ap.radix, ap.radix + ap.nst));
   return it == p->tws_off.end() ? nullptr : reinterpret_cast<const float2*>(p->d_state + it->second);
@@ -479,7 +485,7 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
       p->rplan = AxisPlan{};
       if (real_plan(Lh, p->nelems, p->rplan, width)) {
         p->rplan.width = width;
-        add_stage_table(p, std::vector<int>(p->rplan.radix, p->rplan.radix + p->rplan.nst));
+        add_row_table(p, p->rplan);
         if (!p->tw_off.count(Lh)) p->tw_off[Lh] = image_add(p, nullptr, (size_t)Lh * sizeof(float2));
         if (!p->tw_off.count(2 * Lh)) p->tw_off[2 * Lh] = image_add(p, nullptr, (size_t)2 * Lh * sizeof(float2));
       } else {
@@ -502,7 +508,7 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
         p->aplan[L] = ap;
         p->aplan_s[L] = aps;
         if (!p->tw_off.count(L)) p->tw_off[L] = image_add(p, nullptr, (size_t)L * sizeof(float2));
-        add_stage_table(p, std::vector<int>(ap.radix, ap.radix + ap.nst));
+        add_row_table(p, ap);
         continue;
       }
       if (!is_smooth_235(L) && L <= MAXLEN / 2) {
@@ -517,7 +523,7 @@ int tfft_plan_create(tfft_plan* plan, int ndims, const int64_t* shape, int grid_
       int width = 0;
       if (spec_plan(L, false, p->nelems, ap, width)) {
         ap.width = width;
-        add_stage_table(p, std::vector<int>(ap.radix, ap.radix + ap.nst));
+        add_row_table(p, ap);
       }
       if (spec_plan(L, true, p->nelems, aps, width)) aps.width = width;
       p->aplan[L] = ap;

@@ -271,6 +271,7 @@ bool is_smooth_235(int64_t n);
 bool make_bluestein(tfft_plan p, int N);
 BlueArgs blue_args(tfft_plan p, int N);
 void add_stage_table(tfft_plan p, std::vector<int> radices);
+void add_row_table(tfft_plan p, const AxisPlan& ap);
 const float2* stage_table(tfft_plan p, const AxisPlan& ap);
 int check_ptr(const void* ptr, const char* name);
 int check_bound(tfft_plan p);

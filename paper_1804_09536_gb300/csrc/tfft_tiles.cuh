@@ -68,8 +68,8 @@ __device__ __forceinline__ bool bf_exists(int jt, int q) {
   else return jt + q * T < L / R;
 }
 
-// Offset of stage s in a plan's stage table (launch_stage_twiddles): stages
-// 1 .. s - 1 hold (R - 1) Ns entries each.
+// Offset of stage s in a plan's stage table (TwiddleTable): stages 1 .. s - 1
+// hold (R - 1) Ns entries each.
 template <int S, int... Rs>
 __host__ __device__ constexpr int stage_table_at() {
   constexpr int r[] = {Rs...};
@@ -82,14 +82,10 @@ __host__ __device__ constexpr int stage_table_at() {
 }
 
 // Where a contiguous pass reads stage s's twiddles (spec_stage's OFF): the
-// stage table, except for 512 and 1024 in two stages, which are no faster with
-// it (512^3 pass 0.310 ms either way; 1024 x 64 x 1024 165 us from the roots,
-// 172 from the table).  With it: 2048 50 -> 34 us, 240 24.6 -> 22.5 us,
-// Bluestein 333 59 -> 53 us.
+// stage table, or -1 for the roots (reads_stage_table).
 template <int S, int... Rs>
 __host__ __device__ constexpr int stage_table_off() {
-  constexpr int r[] = {Rs...};
-  return r[0] == 32 && sizeof...(Rs) == 2 ? -1 : stage_table_at<S, Rs...>();
+  return reads_stage_table(sizeof...(Rs), radix_at<0, Rs...>()) ? stage_table_at<S, Rs...>() : -1;
 }
 
 // Twiddle (stage span Ns > 1) and size-R butterflies of a thread's work items.

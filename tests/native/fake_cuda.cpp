@@ -1,7 +1,8 @@
 // A CUDA runtime on host memory (test infrastructure): linked in place of cudart with the library's
 // own objects, it runs the whole host path -- plans, dispatch rules, launch set-up -- without a GPU.
 // Device memory is host memory, kernels do not run, and every launch is recorded with its kernel's
-// name, its grid and, for strided passes, the column blocks it would read.
+// name, its grid and the table it would read: a strided pass's column blocks, a contiguous one's
+// stage table.
 #include <cuda.h>
 #include <cxxabi.h>
 
@@ -39,8 +40,10 @@ cudaError_t record(const void* func, dim3 grid, dim3 block, void** args) {
     cb = reinterpret_cast<unsigned long long>(a.colblocks);
     ncb = a.ncolblocks;
     merged = a.merged_blocks;
+  } else if (name.find("k_contig_spec") != std::string::npos) {
+    cb = reinterpret_cast<unsigned long long>(static_cast<const tfft::ContigArgs*>(args[0])->tws);
   }
-  std::snprintf(line, sizeof line, "%u|%u|%llu|%lld|%lld|", grid.x, block.x * block.y, cb, ncb, merged);
+  std::snprintf(line, sizeof line, "%u|%u|%u|%llu|%lld|%lld|", grid.x, grid.y, block.x * block.y, cb, ncb, merged);
   g_log += line + name + "\n";
   return cudaSuccess;
 }
@@ -57,7 +60,7 @@ int g_token;
 }  // namespace
 
 extern "C" {
-// The launches since the last call, one per line: grid|threads|column blocks|their number|merged blocks|kernel.
+// The launches since the last call, one per line: grid x|grid y|threads|table|column blocks|merged blocks|kernel.
 int fake_launches(char* out, int n) {
   const int len = (int)g_log.size();
   if (len < n) std::memcpy(out, g_log.c_str(), len + 1);

@@ -57,17 +57,19 @@ class Fake:
         assert lib.tfft_plan_state_bytes(self.h, ctypes.byref(nb)) == 0
         self.state = _aligned(nb.value)
         assert lib.tfft_plan_bind(self.h, self.state.ctypes.data, nb.value, None) == 0
-        self.launches()
+        (twiddles,) = self.launches()  # one launch makes every twiddle table, one per grid row
+        assert "k_twiddles" in twiddles[0]
+        self.tables = twiddles[2]
 
     def __del__(self):
         self.lib.tfft_plan_destroy(self.h)
 
     def launches(self):
-        """(kernel, grid, threads, column block address, their number, merged blocks) since the last call."""
+        """(kernel, grid x, grid y, threads, table address, number of column blocks, merged blocks) since the last call."""
         buf = ctypes.create_string_buffer(1 << 16)
         assert self.lib.fake_launches(buf, len(buf)) < len(buf)
-        rows = [r.split("|", 5) for r in buf.value.decode().splitlines()]
-        return [(r[5], *map(int, r[:5])) for r in rows]
+        rows = [r.split("|", 6) for r in buf.value.decode().splitlines()]
+        return [(r[6], *map(int, r[:6])) for r in rows]
 
     def execute(self, sign=-1, events=False):
         """The launches of one call on distinct buffers (no kernel runs)."""
@@ -92,7 +94,7 @@ class Fake:
 
     def column_blocks(self, launch):
         """The column blocks a strided launch reads, which have to lie in the state; None where it reads none."""
-        kernel, _, _, addr, n, merged = launch
+        kernel, _, _, _, addr, n, _ = launch
         if "strided" not in kernel or "k_strided_merged" in kernel or "RankGroupTiles" in kernel:
             return None
         lo = self.state.ctypes.data
@@ -177,3 +179,15 @@ def test_tuning_variable(lib, monkeypatch, ask, threads):
     p = Fake(lib, (32, 512, 64), (2, 2))
     kernels = [k for k, *_ in p.execute() if "k_strided_tma<512" in k]
     assert kernels and f"k_strided_tma<512, {threads}, 16," in kernels[0], kernels
+
+
+@pytest.mark.parametrize("L,tables", [(240, 2), (256, 2), (512, 1), (1024, 1), (2048, 2), (20, 1)])
+def test_stage_tables_made_are_read(lib, L, tables):
+    """A contiguous pass has a stage table in the state when its kernel reads one, and only then;
+    512 and 1024 read the roots, 20 has no compiled row."""
+    p = Fake(lib, (L,), ())
+    assert p.tables == tables
+    (launch,) = p.execute()
+    assert ("k_contig_spec" in launch[0]) == (L != 20)
+    at = launch[4] - p.state.ctypes.data
+    assert 0 <= at and at + 8 * L <= p.state.size if tables == 2 else launch[4] == 0
