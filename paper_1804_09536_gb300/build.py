@@ -20,8 +20,8 @@ LIB = os.path.join(PKG, "libtfft.so")
 
 SOURCES = ["tfft_kernels.cu", "tfft_spec.cu", "tfft_spec_real.cu", "tfft_tma.cu", "tfft_noalloc.cu", "tfft_pointwise.cu", "tfft_batch.cu", "tfft_tc.cu", "tfft_tc_strided.cu", "tfft_blue.cu", "tfft_plan.cpp", "tfft_exchange.cpp",
            "tfft_tmageo.cpp", "tfft_exec.cpp", "tfft_hostio.cpp", "tfft_batch_host.cpp"]
-# the specialised passes, one object per part of their table (kSpecParts in tfft_spec_pass.cuh)
-PARTS = {"tfft_spec_part.cu": [("TFFT_SPEC_PART", k) for k in range(11)]}
+# the specialised passes, one object per part of their table (kSpecParts in tfft_spec_pass.cuh; no row is in part 0)
+PARTS = {"tfft_spec_part.cu": [("TFFT_SPEC_PART", k) for k in range(1, 11)]}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

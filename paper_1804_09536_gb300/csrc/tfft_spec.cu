@@ -1,5 +1,6 @@
 // Plans and dispatch of the compile-time specialised passes: the row of a
 // length in tfft_spec_table.h and the translation unit that compiled it.
+#include "tfft_blue.cuh"
 #include "tfft_spec_pass.cuh"
 
 namespace tfft {
@@ -13,6 +14,15 @@ struct SpecRow {
 #define X(L, T, W, MB, ...) {L, T, W, (int)(sizeof((int[]){__VA_ARGS__}) / sizeof(int)), {__VA_ARGS__}},
 const SpecRow kContigRows[] = {TFFT_CONTIG_LINES(X)};
 const SpecRow kStridedRows[] = {TFFT_STRIDED_LINES(X)};
+#undef X
+
+// every row has a part that is built
+#define X(L, ...) static_assert(L % spec::kSpecParts != 0);
+TFFT_CONTIG_LINES(X)
+TFFT_STRIDED_LINES(X)
+TFFT_BLUE_CONTIG(X)
+TFFT_BLUE_STRIDED(X)
+TFFT_RADER_STRIDED(X)
 #undef X
 
 bool row_plan(const SpecRow& r, AxisPlan& ap, int& width) {

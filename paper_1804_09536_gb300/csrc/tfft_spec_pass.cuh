@@ -157,13 +157,13 @@ cudaError_t run_strided(const StridedArgs& a, cudaStream_t s) {
 
 #undef TFFT_ALLOW_SMEM
 
-// The rows are compiled in kSpecParts translation units (tfft_spec_part.cu),
-// row L in part L mod kSpecParts (a prime above 7 spreads the 2/3/5/7 lengths
-// evenly).
+// The rows are compiled in kSpecParts - 1 translation units (tfft_spec_part.cu),
+// row L in part L mod kSpecParts.  With a prime above 7 the 2/3/5/7 lengths
+// spread over the other remainders, and none is in part 0, which is not built.
 constexpr int kSpecParts = 11;
 
 // calls f(integral_constant<P>) for P == p
-template <int P = 0, class F>
+template <int P = 1, class F>
 cudaError_t with_part(int p, F&& f) {
   if constexpr (P < kSpecParts)
     return p == P ? f(std::integral_constant<int, P>{}) : with_part<P + 1>(p, f);
