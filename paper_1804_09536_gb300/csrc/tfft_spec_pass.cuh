@@ -112,23 +112,14 @@ cudaError_t run_strided_tiles(K kern, const StridedArgs& a, size_t smem, int64_t
 
 template <int L, int T, int W, int MB, bool CHAIN, int... Rs>
 cudaError_t run_strided(const StridedArgs& a, cudaStream_t s) {
-  // Gathering passes, where the two placing warps are a small part of the CTA
-  // (256 threads; 180 x 200 x 240, whose 200 runs five warps, 149 -> 154 us).
-  // Rows of four CTAs per SM always gain (128^4 0.70 -> 0.674 ms per pass, 240
-  // x 240 x 256 on 4 x 4 54 -> 50 us, on 3 x 5 63 -> 61).  The others do where
-  // every stage occupies every thread (320 = 16.20 on 20 threads loses, 58 ->
-  // 62 us at 320 x 320 x 128, 384 = 16.24 on 24 214 -> 224 at 384^3) and the
-  // column blocks are whole (512^3 on 3 x 4 436 -> 426 us, 768 x 768 x 128 326
-  // -> 304); with partial blocks, whose tiles have less to hide the placing
-  // behind, only two stages of at most 20 values do (400^3 on 3 x 5 228 -> 212;
-  // but 512^3 on 1 x 3 514 -> 541, 1024 x 1024 x 256 on 3 x 5 1209 -> 1342).
-  // Or the pass is chained, when its set-up runs before the wait (100 x 150 x
-  // 180 63.0 -> 60.3, 96 x 200 x 96 40.7 -> 39.2; shorter lines gain nothing:
-  // 60 x 72 x 100 19.2 -> 19.5).
-  if constexpr (!CHAIN && L <= 1024) {
-    constexpr bool busy = ((L / Rs >= T) && ...), small = sizeof...(Rs) == 2 && L <= 20 * T;
+  // Gathering tiles: in chained calls from 96 rows on, where their set-up runs
+  // before the wait (100 x 150 x 180 63.0 -> 60.3 us, 96 x 200 x 96 40.7 ->
+  // 39.2; shorter lines gain nothing: 60 x 72 x 100 19.2 -> 19.5), otherwise
+  // for the rows that gain from them (gather_blocks).
+  constexpr int blocks = gather_blocks(L);
+  if constexpr (!CHAIN && L <= 1024 && (L >= 96 || blocks != kGatherNone)) {
     const bool whole = a.ncolblocks * W == a.lin.N[a.d - 1];
-    const bool gains = W * T >= 256 && (MB >= 4 || (busy && (small || whole)));
+    const bool gains = blocks == kGatherAny || (blocks == kGatherWhole && whole);
     if (a.merged_blocks == 0 && (gains || (a.chained && L >= 96)) &&
         a.lin.Mx[a.axis] <= kGatherParts && a.lout.Mx[a.axis] <= kGatherParts) {
       static PerDevice<cudaError_t> attr_cache;

@@ -40,3 +40,23 @@ def test_column_blocks(cuda_device, shape, grid):
     assert rel_l2(y.cpu().numpy(), R.scatter(np.fft.fftn(x.astype(np.complex128)) / x.size, grid, len(grid))) <= RTOL_FP32
     assert np.array_equal(bits(y), bits(p.forward(to_dev(b0, cuda_device), mode="unfused")))
     assert rel_l2(p.inverse(y).cpu().numpy(), b0) <= RTOL_FP32
+
+
+@pytest.mark.parametrize("L", [120, 224, 324, 441, 490, 784, 800, 864, 875, 900, 980, 1008])
+def test_row_tables_and_gathering_agree(cuda_device, L):
+    """Rows that gather only in chained calls: a call with launch events is not chained and runs row tables."""
+    import torch
+    from paper_1804_09536_gb300.plan import Plan
+    for shape, grid in (((5, L, 64), (3, 2)), ((4, L, 35), (1, 3))):
+        x = inputs.uniform_complex(shape, seed=L).numpy()
+        p = Plan(shape, grid, device=cuda_device, tma=False)
+        for sign in (-1, 1):
+            b = to_dev(R.scatter(x, grid, 0 if sign < 0 else 2), cuda_device)
+            want = (p.forward if sign < 0 else p.inverse)(b.clone())
+            events = [torch.cuda.Event(enable_timing=True) for _ in range(p.num_launches(sign) + 1)]
+            p.set_launch_events(events)
+            got = (p.forward if sign < 0 else p.inverse)(b)
+            p.set_launch_events([])
+            f = np.fft.fftn(x.astype(np.complex128)) / x.size if sign < 0 else np.fft.ifftn(x.astype(np.complex128)) * x.size
+            assert rel_l2(got.cpu().numpy(), R.scatter(f, grid, 2 if sign < 0 else 0)) <= RTOL_FP32, (shape, sign)
+            assert np.array_equal(bits(got), bits(want)), (shape, sign)

@@ -191,3 +191,16 @@ def test_stage_tables_made_are_read(lib, L, tables):
     assert ("k_contig_spec" in launch[0]) == (L != 20)
     at = launch[4] - p.state.ctypes.data
     assert 0 <= at and at + 8 * L <= p.state.size if tables == 2 else launch[4] == 0
+
+
+@pytest.mark.parametrize("L,whole,partial", [(64, True, True), (160, True, True), (240, True, True), (400, True, True),
+                                             (245, True, False), (560, True, False), (1024, True, False),
+                                             (60, False, False), (120, False, False), (224, False, False),
+                                             (324, False, False), (490, False, False), (784, False, False),
+                                             (864, False, False), (1008, False, False)])
+def test_gathering_rows(lib, L, whole, partial):
+    """Outside chained calls a cut pass runs gathering tiles where its row gains from them."""
+    for K, want in ((128, whole), (127, partial)):
+        p = Fake(lib, ((1 << 23) // (L * K) + 1, L, K), (2, 2), flags=8)  # too large to chain, no TMA
+        kernels = [k for k, *_ in p.execute() if f"strided_spec<{L}," in k or f"strided_gather<{L}," in k]
+        assert len(kernels) == 1 and ("gather" in kernels[0]) == want, (K, kernels)
