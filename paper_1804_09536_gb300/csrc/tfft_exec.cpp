@@ -561,10 +561,18 @@ int run_steps_cached(tfft_plan p, const tfft_plan_s::GraphKey& k, const std::fun
       --live;
     }
     cudaGraph_t g = nullptr;
+    const std::vector<Step> steps = make_steps();
     cudaError_t ce = cudaStreamBeginCapture(p->capture_stream, cudaStreamCaptureModeRelaxed);
     int rc = TFFT_OK;
     if (ce == cudaSuccess) {
-      rc = run_steps(p, make_steps(), bufs, p->capture_stream);
+      try {
+        rc = run_steps(p, steps, bufs, p->capture_stream);
+      } catch (...) {  // out of host memory: no capture stays open
+        cudaStreamEndCapture(p->capture_stream, &g);
+        if (g) cudaGraphDestroy(g);
+        cudaGetLastError();
+        throw;
+      }
       ce = cudaStreamEndCapture(p->capture_stream, &g);
     }
     if (rc == TFFT_OK && ce == cudaSuccess && g) ce = cudaGraphInstantiate(&e.exec, g, 0);
@@ -574,7 +582,7 @@ int run_steps_cached(tfft_plan p, const tfft_plan_s::GraphKey& k, const std::fun
       cudaGetLastError();
       e.exec = nullptr;
       e.calls = -(1 << 30);
-      return run_steps(p, make_steps(), bufs, st);
+      return run_steps(p, steps, bufs, st);
     }
   }
   if (!e.exec) return run_steps(p, make_steps(), bufs, st);

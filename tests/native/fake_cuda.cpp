@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <new>
 #include <string>
 
 #include "tfft_internal.h"
@@ -30,7 +31,11 @@ std::string demangled(const char* name) {
   return s;
 }
 
+bool g_graphs = false, g_capturing = false;  // captures refused, unless asked for
+int g_fail = 0;                              // launches until one runs out of host memory
+
 cudaError_t record(const void* func, dim3 grid, dim3 block, void** args) {
+  if (g_fail > 0 && --g_fail == 0) throw std::bad_alloc();
   const std::string& name = kernels()[func];
   char line[256];
   unsigned long long cb = 0;
@@ -67,6 +72,10 @@ int fake_launches(char* out, int n) {
   g_log.clear();
   return len;
 }
+
+void fake_graphs(int on) { g_graphs = on != 0; }
+int fake_capturing() { return g_capturing; }
+void fake_fail_launch(int n) { g_fail = n; }
 
 void** __cudaRegisterFatBinary(void*) { return reinterpret_cast<void**>(&g_token); }
 void __cudaRegisterFatBinaryEnd(void**) {}
@@ -121,17 +130,35 @@ cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
   return cudaSuccess;
 }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t*, unsigned) { return cudaErrorNotSupported; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
+  *s = reinterpret_cast<cudaStream_t>(&g_token);
+  return cudaSuccess;
+}
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
-  *s = cudaStreamCaptureStatusActive;  // launches go directly, never through the graph cache
+  // a caller's capture: launches go directly, not through the graph cache
+  *s = g_graphs ? cudaStreamCaptureStatusNone : cudaStreamCaptureStatusActive;
   return cudaSuccess;
 }
-cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaErrorNotSupported; }
-cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t*) { return cudaErrorNotSupported; }
-cudaError_t cudaGraphInstantiate(cudaGraphExec_t*, cudaGraph_t, unsigned long long) { return cudaErrorNotSupported; }
-cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaErrorNotSupported; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) {
+  if (g_capturing) return cudaErrorIllegalState;
+  g_capturing = true;
+  return cudaSuccess;
+}
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) {
+  *g = g_capturing ? reinterpret_cast<cudaGraph_t>(&g_token) : nullptr;
+  g_capturing = false;
+  return cudaSuccess;
+}
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t, unsigned long long) {
+  *x = reinterpret_cast<cudaGraphExec_t>(&g_token);
+  return cudaSuccess;
+}
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) {
+  g_log += "0|0|0|0|-1|0|graph\n";
+  return cudaSuccess;
+}
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t*) { return cudaErrorNotSupported; }

@@ -204,3 +204,24 @@ def test_gathering_rows(lib, L, whole, partial):
         p = Fake(lib, ((1 << 23) // (L * K) + 1, L, K), (2, 2), flags=8)  # too large to chain, no TMA
         kernels = [k for k, *_ in p.execute() if f"strided_spec<{L}," in k or f"strided_gather<{L}," in k]
         assert len(kernels) == 1 and ("gather" in kernels[0]) == want, (K, kernels)
+
+
+def test_capture_ends_when_a_launch_throws(lib):
+    """The second identical call captures its launches; one that runs out of host memory there leaves
+    no capture open, and the next call captures and replays as usual."""
+    p = Fake(lib, (32, 32, 32), (2, 2))
+    lib.fake_graphs(1)
+    try:
+        assert len(p.execute()) == 3
+        lib.fake_fail_launch(2)
+        nb = ctypes.c_size_t()
+        assert lib.tfft_plan_workspace_bytes(p.h, 0, 1, ctypes.byref(nb)) == 0
+        at = 1 << 40
+        assert lib.tfft_execute(p.h, -1, 0, at, 2 * at, 3 * at, nb.value, None) != 0
+        assert not lib.fake_capturing()
+        p.launches()
+        assert [k for k, *_ in p.execute()][-1] == "graph"
+        assert [k for k, *_ in p.execute()] == ["graph"]
+    finally:
+        lib.fake_fail_launch(0)
+        lib.fake_graphs(0)
