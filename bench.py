@@ -303,9 +303,9 @@ def run_ours(args):
                      tma=not args.no_tma, shape=(512, 512, 512), grid=(4, 8))
 
     # the 4-D case: 128^4 on a 3-D virtual grid
-    # the appendix's shape with non-2/3/5 lengths (127 by Bluestein) on a 3 x 4 grid
+    # the appendix's shape with non-2/3/5 lengths (127 by Rader) on a 3 x 4 grid
     appa = appendix_a(plan_cls=Plan, dev=dev, steps=max(3, min(args.steps, 20)), barrier=barrier)
-    # the same kind of axis (127, Bluestein) in an array larger than L2
+    # the same kind of axis (127, Rader) in an array larger than L2
     blue = appendix_a(plan_cls=Plan, dev=dev, steps=max(3, min(args.steps, 20)), barrier=barrier,
                       shape=(512, 127, 512), grid=(4, 4))
     fd = fourd_128(plan_cls=Plan, dev=dev, steps=max(3, min(args.steps, 20)), barrier=barrier,
@@ -704,7 +704,7 @@ def r2c_slab(plan_cls, dev, steps, barrier, tma=True, shape=(256, 256, 256), gri
 
 def appendix_a(plan_cls, dev, steps, barrier, shape=(42, 127, 256), grid=(3, 4)):
     """App. A's 42 x 127 x 256 c2c on a 3 x 4 grid (42 = 2.3.7 and the prime 127 by
-    Bluestein's convolution form), or another shape: fused forward + inverse,
+    a convolution), or another shape: fused forward + inverse,
     per-launch times and GB/s of algorithmic bytes (16 B per element per pass)."""
     import torch
     from paper_1804_09536_gb300 import inputs
@@ -740,8 +740,8 @@ def appendix_a(plan_cls, dev, steps, barrier, shape=(42, 127, 256), grid=(3, 4))
     peak, _ = _peaks()
     nbytes = sum(nb for _, nb in p.launch_info(-1) + p.launch_info(+1))
     mib = 8 * n / 2**20
-    return {"workload": f"{'x'.join(map(str, shape))} c2c complex64 (lengths without a 2/3/5 factorisation by "
-                        f"Bluestein), virtual grid {'x'.join(map(str, grid))}, forward+inverse, fused; "
+    return {"workload": f"{'x'.join(map(str, shape))} c2c complex64 (lengths without a 2/3/5 "
+                        f"factorisation), virtual grid {'x'.join(map(str, grid))}, forward+inverse, fused; "
                         f"{mib:.1f} MiB per stage buffer ({'L2-resident' if 8 * n < 129e6 else 'larger than L2'})",
             "ms_per_step": round(ms, 4), "hbm_frac": round(nbytes / (ms * 1e-3) / 1e9 / peak, 4),
             "graph_ms_per_step": round(ms_graph, 4),

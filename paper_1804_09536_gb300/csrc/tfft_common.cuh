@@ -433,8 +433,9 @@ TFFT_HD int stockham_tw_index(int j, int Ns, int R, int r, int L) {
 // int moved those and cost the TMA-staged passes 0.6 % (512^3 1948 -> 1960 us).
 struct AxisPlan {
   int L;           // transform length
-  int E;           // elements per thread (every radix divides E)
-  int T;           // threads per line = L / E
+  int E;           // runtime-radix kernels: elements per thread (every radix divides E), 0 = generic;
+                   // compiled rows: ceil(L / T), but a thread holds emax<L, T, radices>() values
+  int T;           // threads per line
   int nst;         // number of radix stages
   uint64_t code;   // radix of stage s = (code >> 5 s) & 31
   int spec;        // 1: a compile-time specialised kernel exists for this plan

@@ -54,9 +54,9 @@ struct ContigArgs {
   int chained;       // kChain* bits, see launch_chained
 };
 
-// Bluestein's algorithm for a line length N without a 2/3/5 factorisation:
-// the DFT as a circular convolution of length M (a power of two >= 2N - 1)
-// with a chirp, done with two length-M FFTs.
+// Bluestein's algorithm for a line length N without a plan of its own: the DFT
+// as a circular convolution with a chirp, done with two FFTs of length M >=
+// 2N - 1 (a compiled length, or a power of two for the runtime kernels).
 struct BlueArgs {
   int N, M;
   AxisPlan apm;          // length-M FFT plan (shared-memory stages)

@@ -132,7 +132,13 @@ cudaError_t run_strided(const StridedArgs& a, cudaStream_t s) {
     if (a.chained) return run_strided<L, T, W, MB, true, Rs...>(a, s);
   const int chained = CHAIN ? a.chained : 0;
   // in-place leading-axis passes run merged columns (400^3 on 4 x 4 0.250 ->
-  // 0.174 ms, 240^3 on 4 x 8 51 -> 41 us, 180 x 200 x 240 34.8 -> 24.6 us)
+  // 0.174 ms, 240^3 on 4 x 8 51 -> 41 us, 180 x 200 x 240 34.8 -> 24.6 us; over
+  // every row at 2^24 elements 1.14 in the geometric mean).  The merged kernel
+  // takes the launch bounds of the row-table kernel but forms every row's
+  // address from the run-time `inner`: 57 of its 188 instantiations spill, 68
+  // bytes at most at the powers of two up to 512, 96 132-140, 144 128-144, 288
+  // and 576 124.  The worst lose to the row tables: 81 (180 bytes) 55 -> 60 us,
+  // 243 (212) 65 -> 70, 392 (204) 64 -> 68; 864, 972 and 1000 lose 3-4 %.
   if (a.merged_blocks > 0) {
     static PerDevice<cudaError_t> attr_cache;
     static PerDevice<int64_t> slots_cache;
